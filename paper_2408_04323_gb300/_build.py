@@ -15,7 +15,7 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libscoot.so")
-SOURCES = ["context.cu", "host_prep.cpp", "compact.cu", "prune_rf.cu", "score.cu", "topq.cu", "fantasy.cu", "pareto.cu",
+SOURCES = ["context.cu", "host_prep.cpp", "compact.cu", "prune_rf.cu", "score.cu", "ehvi.cu", "topq.cu", "fantasy.cu", "pareto.cu",
            "sobol.cu", "rf_train.cu",
            "gp_device.cu", "round_state.cpp", "probes.cu", "posterior_tc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -130,6 +130,43 @@ __device__ __forceinline__ float ehvi_value(const float* mu, const float* sd, co
     return total * (1.0f / (float)n_mc);
 }
 
+// Partial EHVI sum of one candidate over the sample chunks first, first +
+// stride, ... (chunks of eight samples, padding samples at -inf); boxes as
+// staged by stage_boxes.
+template <int M>
+__device__ __forceinline__ float ehvi_partial(const float* mu, const float* sd, const float4* blo, const float4* bhi,
+                                             int n_boxes, const float4* eps, int n_mc, int first, int stride) {
+    constexpr int kCh = 8;
+    float total = 0.0f;
+    for (int s0 = first * kCh; s0 < n_mc; s0 += stride * kCh) {
+        float y[kCh][M], acc[kCh];
+#pragma unroll
+        for (int k = 0; k < kCh; ++k) {
+            acc[k] = 0.0f;
+            const bool in = s0 + k < n_mc;
+            const float4 e = in ? eps[s0 + k] : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float ev[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+            for (int j = 0; j < M; ++j) y[k][j] = in ? fmaf(sd[j], ev[j], mu[j]) : -INFINITY;
+        }
+        for (int b = 0; b < n_boxes; ++b) {
+            const float4 lo4 = blo[b], hi4 = bhi[b];
+            const float lo[4] = {lo4.x, lo4.y, lo4.z, lo4.w};
+            const float hi[4] = {hi4.x, hi4.y, hi4.z, hi4.w};
+#pragma unroll
+            for (int k = 0; k < kCh; ++k) {
+                float p = fmaxf(fminf(y[k][0], hi[0]) - lo[0], 0.0f);
+#pragma unroll
+                for (int j = 1; j < M; ++j) p *= fmaxf(fminf(y[k][j], hi[j]) - lo[j], 0.0f);
+                acc[k] += p;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kCh; ++k) total += acc[k];
+    }
+    return total;
+}
+
 // Width that stands in for an unbounded side of a box on the first M-1
 // objectives: a power of two, so scaling by it and by its inverse is exact;
 // valid while every sample lies within 2^40 of the box's lower corner.

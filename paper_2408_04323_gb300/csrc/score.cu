@@ -67,43 +67,6 @@ struct ScoreArgs {
     uint32_t* err;                // device error word
 };
 
-// Partial EHVI sum of one candidate over the sample chunks first, first +
-// stride, ... (chunks of eight samples, padding samples at -inf); boxes as
-// staged by stage_boxes.
-template <int M>
-__device__ __forceinline__ float ehvi_partial(const float* mu, const float* sd, const float4* blo, const float4* bhi,
-                                             int n_boxes, const float4* eps, int n_mc, int first, int stride) {
-    constexpr int kCh = 8;
-    float total = 0.0f;
-    for (int s0 = first * kCh; s0 < n_mc; s0 += stride * kCh) {
-        float y[kCh][M], acc[kCh];
-#pragma unroll
-        for (int k = 0; k < kCh; ++k) {
-            acc[k] = 0.0f;
-            const bool in = s0 + k < n_mc;
-            const float4 e = in ? eps[s0 + k] : make_float4(0.f, 0.f, 0.f, 0.f);
-            const float ev[4] = {e.x, e.y, e.z, e.w};
-#pragma unroll
-            for (int j = 0; j < M; ++j) y[k][j] = in ? fmaf(sd[j], ev[j], mu[j]) : -INFINITY;
-        }
-        for (int b = 0; b < n_boxes; ++b) {
-            const float4 lo4 = blo[b], hi4 = bhi[b];
-            const float lo[4] = {lo4.x, lo4.y, lo4.z, lo4.w};
-            const float hi[4] = {hi4.x, hi4.y, hi4.z, hi4.w};
-#pragma unroll
-            for (int k = 0; k < kCh; ++k) {
-                float p = fmaxf(fminf(y[k][0], hi[0]) - lo[0], 0.0f);
-#pragma unroll
-                for (int j = 1; j < M; ++j) p *= fmaxf(fminf(y[k][j], hi[j]) - lo[j], 0.0f);
-                acc[k] += p;
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < kCh; ++k) total += acc[k];
-    }
-    return total;
-}
-
 // Asynchronous copy of one half of a 32 x 64 tile of L^{-1} (16 columns x 64
 // rows, 4 KiB, contiguous in the host's transposed tile layout and 16-byte
 // aligned at both ends) into shared memory: each of the 128 threads moves two
@@ -745,6 +708,54 @@ scoot_status tc_direct(scoot_ctx* ctx, const ScoreArgs& a, const uint8_t* mask, 
     return scoot_posterior_tc(ctx, t, DO, st);
 }
 
+// The route of scoot_score_ehvi through the tensor cores: the posterior's
+// moments by list position into the workspace, then the EHVI of ehvi.cu.
+// Workspace: the compacted list (when masked), the split copy of L^{-1}, the
+// moments and the EHVI's scratch, reserved whole before the list is written.
+// *used as for tc_direct.
+scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* used) {
+    *used = false;
+    const int M = a.n_obj;
+    if (!ctx->tensor_cores || a.n_rb * kRB > kMaxNpadTc) return SCOOT_OK;
+    // One row block (n <= 64) is too little for the tensor cores' pipeline:
+    // there the fused kernel stays ahead (n = 64, M = 2, 2^18 candidates 134 us
+    // against 160) unless the walk saves more (M = 3, 132 boxes, 2^18: 444 us
+    // against 648; 2^15: 113 against 103).
+    // Up to 128 observations it takes 16384 candidates (n = 100, M = 2: 4096
+    // candidates 41 us fused against 43, 16384 48 against 45, 65536 92 against
+    // 69); beyond, the fused kernel loses from 2048 on (n = 200: 78 against 58).
+    if (a.n_rb == 1 && !(a.n >= 65536 && scoot_ehvi_walks(M, a.n, a.n_boxes, a.n_mc))) return SCOOT_OK;
+    if (a.n_rb == 2 && a.n < 16384) return SCOOT_OK;
+    ScootTcArgs t = tc_args(ctx, a, M);
+    const int DO = tc_do(a);
+    if (!scoot_tc_supported(ctx, t, DO)) return SCOOT_OK;
+    *used = true;
+    const size_t list_bytes = a.mask ? ((256 + (size_t)a.n * 4 + 255) & ~(size_t)255) : 0;
+    const size_t split_bytes = ((size_t)scoot_tc_bsplit_bytes(t.n_pad, M) + 255) & ~(size_t)255;
+    const size_t moment_bytes = ((size_t)M * a.n * 4 + 255) & ~(size_t)255;
+    scoot_status s = scoot_workspace(ctx, list_bytes + split_bytes + 2 * moment_bytes +
+                                              scoot_ehvi_work_bytes(M, a.n, a.n_boxes, a.n_mc));
+    if (s != SCOOT_OK) return s;
+    if (a.mask) {
+        ScootList lst;
+        if ((s = scoot_compact(ctx, a.mask, a.n, reinterpret_cast<uint32_t*>(a.acq), 0xFF800000u, st, &lst)) != SCOOT_OK)
+            return s;
+        t.list = lst.list;
+        t.n_list = lst.count;
+    }
+    char* ws = static_cast<char*>(ctx->ws) + list_bytes;
+    t.cand = a.cand;
+    t.n = a.n;
+    t.ld = a.ld;
+    t.bsplit = reinterpret_cast<uint8_t*>(ws);
+    t.mean = reinterpret_cast<float*>(ws + split_bytes);
+    t.var = reinterpret_cast<float*>(ws + split_bytes + moment_bytes);
+    t.ldo = a.n;
+    if ((s = scoot_posterior_tc(ctx, t, DO, st)) != SCOOT_OK) return s;
+    return scoot_ehvi_listed(ctx, M, t.mean, t.var, a.n, a.n, t.list, t.n_list, a.box_lo, a.box_hi, a.n_boxes, a.eps,
+                             a.n_mc, ws + split_bytes + 2 * moment_bytes, a.acq, st);
+}
+
 }  // namespace
 
 scoot_status scoot_posterior_whitened(scoot_ctx* ctx, const scoot_gp_layout* L, const void* state,
@@ -1043,6 +1054,9 @@ scoot_status scoot_score_ehvi(scoot_ctx* ctx, const scoot_gp_layout* L, const vo
     a.n_boxes = n_boxes;
     a.eps = eps;
     a.n_mc = n_mc;
+    bool used = false;
+    s = tc_ehvi(ctx, a, static_cast<cudaStream_t>(stream), &used);
+    if (used || s != SCOOT_OK) return s;
     return dispatch_m<kEHVI>(ctx, a, L->n_obj, static_cast<cudaStream_t>(stream));
 }
 
