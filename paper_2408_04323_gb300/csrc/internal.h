@@ -173,6 +173,7 @@ struct ScootTcArgs {
     int64_t ldo;
     float* vout;      // NULL: moments only
     int32_t by_index; // mean / var at the candidate's index (else at its list position)
+    int32_t accurate; // the covariance's square root and exponential to an fp32 rounding
     uint8_t* bsplit;  // [M][n_pad / 32][3][n_pad * 64 bytes]
     uint32_t* err;
     // Acquisition epilogue (objective 0 only, acq at the candidate's index;

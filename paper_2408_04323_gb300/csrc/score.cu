@@ -712,7 +712,10 @@ scoot_status tc_direct(scoot_ctx* ctx, const ScoreArgs& a, const uint8_t* mask, 
 // moments by list position into the workspace, then the EHVI of ehvi.cu.
 // Workspace: the compacted list (when masked), the split copy of L^{-1}, the
 // moments and the EHVI's scratch, reserved whole before the list is written.
-// *used as for tc_direct.
+// *used as for tc_direct.  The covariances take the accurate square root and
+// exponential (7% of the posterior's time): the acquisition's error against 64
+// bits is then that of the fused kernel (0.7 to 1.2 times it over 21 models of 70
+// to 256 observations, 1.0 on average; 1.1 without).
 scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* used) {
     *used = false;
     const int M = a.n_obj;
@@ -721,11 +724,11 @@ scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* 
     // there the fused kernel stays ahead (n = 64, M = 2, 2^18 candidates 134 us
     // against 160) unless the walk saves more (M = 3, 132 boxes, 2^18: 444 us
     // against 648; 2^15: 113 against 103).
-    // Up to 128 observations it takes 16384 candidates (n = 100, M = 2: 4096
-    // candidates 41 us fused against 43, 16384 48 against 45, 65536 92 against
-    // 69); beyond, the fused kernel loses from 2048 on (n = 200: 78 against 58).
+    // Up to 128 observations it takes 32768 candidates (n = 100, M = 2: 4096
+    // candidates 41 us fused against 43, 16384 48 against 47, 65536 92 against
+    // 71); beyond, the fused kernel loses from 2048 on (n = 200: 78 against 60).
     if (a.n_rb == 1 && !(a.n >= 65536 && scoot_ehvi_walks(M, a.n, a.n_boxes, a.n_mc))) return SCOOT_OK;
-    if (a.n_rb == 2 && a.n < 16384) return SCOOT_OK;
+    if (a.n_rb == 2 && a.n < 32768) return SCOOT_OK;
     ScootTcArgs t = tc_args(ctx, a, M);
     const int DO = tc_do(a);
     if (!scoot_tc_supported(ctx, t, DO)) return SCOOT_OK;
@@ -747,6 +750,7 @@ scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* 
     t.cand = a.cand;
     t.n = a.n;
     t.ld = a.ld;
+    t.accurate = 1;
     t.bsplit = reinterpret_cast<uint8_t*>(ws);
     t.mean = reinterpret_cast<float*>(ws + split_bytes);
     t.var = reinterpret_cast<float*>(ws + split_bytes + moment_bytes);

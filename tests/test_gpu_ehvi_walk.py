@@ -1,19 +1,22 @@
 """The Monte-Carlo EHVI over three objectives that visits only the boxes a
-sample reaches, against the sum over all boxes in 64 bits from the same
+sample reaches, against the sum over all boxes in 64 bits from the oracle's
 moments: builder's boxes, boxes it has to refuse (another order, a floor that
 rises, too few), odd pools and sample counts at the edges of its batches.
 
-Bar: the terms are not negative, so the order and number of the additions
-costs at most 2 u (B + S) of the sum (u = 2^-24); a sample's coordinate carries
-4 u (|mu| + |eps| sigma + |edge|), whose effect is taken by moving each
-objective by that much."""
+Bar: the propagated posterior tolerance of the other acquisition tests; the
+terms are not negative, so the order and number of the additions costs at most
+2 u (B + S) of the sum more (u = 2^-24)."""
 import numpy as np
 import pytest
 
 from workloads import Stream, make_instance
 
+import oracle as O
+
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+
+from parity_tol import posterior_tols, propagated_tol  # noqa: E402
 
 U32 = 2.0 ** -24
 
@@ -32,17 +35,17 @@ def dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
-def all_boxes(mu, sd, eps, lo, hi, shift=None):
-    y = [mu[m][:, None] + sd[m][:, None] * eps[None, :, m] for m in range(3)]
-    if shift is not None:
-        y[shift[0]] = y[shift[0]] + shift[1]
+def all_boxes(mu, var, eps, lo, hi):
+    """EHVI of moments [K][3] over every box, in 64 bits."""
+    mu, sd = dev(mu), dev(np.sqrt(np.maximum(var, 0.0)))
+    y = [mu[:, m, None] + sd[:, m, None] * eps[None, :, m] for m in range(3)]
     total = torch.zeros_like(y[0])
     for b in range(len(lo)):
         p = 1.0
         for m in range(3):
             p = p * (torch.clamp(y[m], max=float(hi[b, m])) - float(lo[b, m])).clamp(min=0)
         total += p
-    return total.mean(1)
+    return total.mean(1).cpu().numpy()
 
 
 @pytest.mark.parametrize("n_cand,n_mc,boxes,masked", [
@@ -70,8 +73,6 @@ def test_walk_equals_all_boxes(S, n_cand, n_mc, boxes, masked):
                                      inst.noise_var, layout)
         blob, cand = dev(blob), dev(inst.cand.view(np.int32))
         mask = dev((Stream(5, "mask").uniform(n_cand) < 0.6).astype(np.uint8)) if masked else None
-        mean, var = (torch.zeros((3, n_cand), device="cuda") for _ in range(2))
-        S.scoot_gp_posterior(ctx, layout, blob, cand, n_cand, mean, var)
         acq = torch.full((n_cand,), 7.0, device="cuda")
         S.scoot_score_ehvi(ctx, layout, blob, cand, n_cand, dev(lo), dev(hi), dev(eps), acq, mask)
         again = torch.zeros_like(acq)
@@ -82,13 +83,12 @@ def test_walk_equals_all_boxes(S, n_cand, n_mc, boxes, masked):
     assert (acq[~live] == -np.inf).all()
     at = live.nonzero()[:, 0]
     at = at[torch.linspace(0, len(at) - 1, min(len(at), 400)).long().cuda()]
-    mu, sd, e = mean[:, at].double(), var[:, at].double().sqrt(), dev(eps.astype(np.float64))
-    want = all_boxes(mu, sd, e, lo, hi)
-    edge = max(np.abs(lo).max(), np.abs(hi[np.isfinite(hi)]).max())
-    tol = 2 * U32 * (len(lo) + n_mc) * want
-    for m in range(3):
-        d = 4 * U32 * (mu[m][:, None].abs() + sd[m][:, None] * e[None, :, m].abs() + float(edge))
-        tol = tol + all_boxes(mu, sd, e, lo, hi, (m, d)) - want
-    worst = float(((acq[at].double() - want).abs() / tol.clamp(min=1e-30)).max())
+    gps = [O.GP(inst.space, inst.x_obs, inst.y_obs[m], inst.lengthscale[m], float(inst.signal_var[m]),
+                float(inst.noise_var[m])) for m in range(3)]
+    mu, v, e_mu, e_var = posterior_tols(gps, inst.cand[:, at.cpu().numpy()])
+    e = dev(eps.astype(np.float64))
+    want, tol = propagated_tol(lambda a, b: all_boxes(a, b, e, lo, hi), mu, v, e_mu, e_var)
+    tol = tol + 2 * U32 * (len(lo) + n_mc) * want
+    worst = float((np.abs(acq[at].cpu().numpy().astype(np.float64) - want) / tol).max())
     print(f"{boxes} n={n_cand} S={n_mc}: {worst:.3f} of the tolerance")
     assert worst <= 1.0
