@@ -1,5 +1,6 @@
 // Known-constraint pruning (Eq. 2) and random-forest probability of
 // feasibility (Eq. 3) over a structure-of-arrays candidate pool.
+#include <algorithm>
 #include <cstring>
 
 #include "internal.h"
@@ -137,16 +138,15 @@ struct RfArgs {
 // (the upper levels are broadcast loads) and each candidate has eight
 // independent walks in flight.  The forest (or one chunk of whole trees at a
 // time) sits in shared memory with chunk-relative child indices; the tile's
-// feature values sit in shared memory as feat[slot][f] with an odd row
-// stride (conflict-free when a warp reads one feature).  The eight partial
+// feature values sit in shared memory as feat[f][slot], so that a lane's reads
+// stay in its own bank whatever features the lanes ask for.  The eight partial
 // vote counts of a candidate are added through shared memory.
 __global__ void __launch_bounds__(kRfThreads)
 rf_kernel(const __grid_constant__ RfArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int fs = a.d | 1;                                                       // odd row stride
     uint2* snodes = reinterpret_cast<uint2*>(smem_raw);                           // chunk nodes
-    float* sfeat = reinterpret_cast<float*>(snodes + a.max_chunk_nodes);          // [kRfCand][fs]
-    uint32_t* svote = reinterpret_cast<uint32_t*>(sfeat + kRfCand * fs);          // [kRfGroups][kRfCand]
+    float* sfeat = reinterpret_cast<float*>(snodes + a.max_chunk_nodes);          // [d][kRfCand]
+    uint32_t* svote = reinterpret_cast<uint32_t*>(sfeat + kRfCand * a.d);         // [kRfGroups][kRfCand]
     int32_t* sroot = reinterpret_cast<int32_t*>(svote + kRfGroups * kRfCand);      // [n_trees]
 
     const int32_t* chunks = reinterpret_cast<const int32_t*>(a.forest + a.off_chunks);
@@ -159,15 +159,15 @@ rf_kernel(const __grid_constant__ RfArgs a) {
     uint32_t feasible = 0;
 
     // Staged node word: x = threshold bits (split) or vote count as a float
-    // (leaf); y = chunk-relative left child in bits 0..15, the feature's byte
-    // offset in a feature row in bits 16..30, bit 31 set for a leaf.
+    // (leaf); y = chunk-relative left child in bits 0..15, the byte offset of
+    // the feature's values in bits 16..30, bit 31 set for a leaf.
     auto stage_chunk = [&](int ch) {
         const int t0 = chunks[ch * 4 + 0], nt = chunks[ch * 4 + 1];
         const int first_node = chunks[ch * 4 + 2], count = chunks[ch * 4 + 3];
         for (int k = tid; k < count; k += kRfThreads) {
             const uint2 g = __ldg(gnodes + first_node + k);
             const uint32_t leaf = (g.y >> 24) & 1u, feat = (g.y >> 16) & 0xffu;
-            snodes[k] = make_uint2(g.x, leaf ? 0x80000000u : ((feat * 4u) << 16) | (g.y & 0xffffu));
+            snodes[k] = make_uint2(g.x, leaf ? 0x80000000u : ((feat * 4u * kRfCand) << 16) | (g.y & 0xffffu));
         }
         for (int k = tid; k < nt; k += kRfThreads) sroot[t0 + k] = roots[t0 + k] - first_node;
     };
@@ -193,12 +193,12 @@ rf_kernel(const __grid_constant__ RfArgs a) {
                     const uint32_t w = __ldg(a.cand + (int64_t)f * a.ld + i);
                     x = ((a.float_cols >> f) & 1u) ? __uint_as_float(w) : (float)(int32_t)w;
                 }
-                sfeat[c * fs + f] = x;
+                sfeat[f * kRfCand + c] = x;
             }
             __syncthreads();
             const int64_t pos = base + slot;
             const bool live = pos < n_work;
-            const char* my = reinterpret_cast<const char*>(sfeat + slot * fs);
+            const char* my = reinterpret_cast<const char*>(sfeat + slot);
             uint32_t vote = 0;
             // The lanes of a warp walk the same tree (for 32 candidates) in
             // lockstep, so the upper levels of the tree are broadcast loads;
@@ -237,6 +237,217 @@ rf_kernel(const __grid_constant__ RfArgs a) {
                     feasible += ok;
                 }
             }
+        }
+    }
+    if (a.count) add_count(a.count, feasible);
+}
+
+// ---------------------------------------------------------------- ranked forests
+//
+// x <= t holds exactly when the number of the forest's distinct thresholds of
+// that feature below x is at most the number below t.  So with every feature
+// value replaced by such a rank plus one, at the top of a word, one comparison of
+// whole words decides, and a node in shared memory is two words that need no
+// arithmetic but a mask:
+//   split: threshold's rank plus one << 19 | feature << 7 (the byte offset of
+//          the feature's 32 values), and the address of the left child;
+//   leaf:  8191 << 19 | its votes (in bits 18..11 and 6..0), and its own
+//          address, so that a walk that has ended stays there.
+// (Thresholds are finite; a NaN feature has the largest rank, 8191, and goes right
+// at every split, as a float comparison does.)
+// The walk is bound by instructions (rf_kernel: 77% of the issue slots, few bank
+// conflicts), which the loop of rf_kernel spends 15 of per visit, with lanes
+// idle that have reached a leaf; this one spends 5 and no branch, with a look
+// every two visits at whether all 32 lanes have ended.  On 2.17 M candidates and 200 trees
+// (11600 nodes) 1.82 ms and 0.03 for the ranking, against 2.76.  Measured and not
+// kept: four-byte nodes (seven to nine instructions a visit, 2.9 ms) and two
+// trees at a time (the longer one's visits and 8-byte gathers fill the shared-
+// memory pipe, 12% slower).
+constexpr int kRankNodes = 16380;         // 13 bits of rank; 131 KB of nodes
+constexpr int kRankThr = 8192;            // distinct thresholds of a feature (at most (nodes - 1) / 2)
+constexpr int kRankVotes = 32767;         // votes of a leaf
+constexpr uint32_t kRankEnd = 8191u << 19;
+constexpr int kRankThreads = 1024;
+constexpr int64_t kRankFrom = 400000000;  // candidates x trees x depth that pay for the ranking
+constexpr int kRankTiles = 4;             // tiles of 32 candidates per block, eight groups of trees each
+constexpr int kRankWalkThreads = kRankTiles * kRfThreads;
+
+struct RankArgs {
+    const char* forest;
+    int64_t off_chunks, off_nodes;
+    int32_t n_chunks, n_nodes;
+    uint2* nodes;      // [n_nodes] ranked nodes, with the child's number for its address
+    float* thr;        // [d][kRankThr] distinct thresholds, increasing
+    int32_t* n_thr;    // [d]
+};
+
+// Block f: the distinct thresholds of feature f, sorted, and the ranked nodes
+// that split on it (block 0 also the leaves).
+__global__ void __launch_bounds__(kRankThreads) rank_forest_kernel(const __grid_constant__ RankArgs a) {
+    __shared__ float key[kRankThr];
+    __shared__ int s_cnt, s_wt[kRankThreads / 32];
+    const int f = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint2* nodes = reinterpret_cast<const uint2*>(a.forest + a.off_nodes);
+    const int4* chunks = reinterpret_cast<const int4*>(a.forest + a.off_chunks);  // .z first node, .w nodes
+    if (tid == 0) s_cnt = 0;
+    __syncthreads();
+    for (int k0 = 0; k0 < a.n_nodes; k0 += kRankThreads) {
+        const int k = k0 + tid;
+        const uint2 g = k < a.n_nodes ? __ldg(nodes + k) : make_uint2(0u, 1u << 24);
+        const bool mine = !((g.y >> 24) & 1u) && (int)((g.y >> 16) & 0xffu) == f;
+        const unsigned b = __ballot_sync(0xffffffffu, mine);
+        int at = 0;
+        if (lane == 0 && b) at = atomicAdd(&s_cnt, __popc(b));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(b & ((1u << lane) - 1u));
+        if (mine && at < kRankThr) key[at] = __uint_as_float(g.x);
+    }
+    __syncthreads();
+    const int cnt = min(s_cnt, kRankThr);
+    int P = 1;
+    while (P < cnt) P *= 2;
+    for (int e = cnt + tid; e < P; e += kRankThreads) key[e] = INFINITY;
+    __syncthreads();
+    for (int k = 2; k <= P; k *= 2)
+        for (int j = k / 2; j > 0; j /= 2) {
+            for (int e = tid; e < P; e += kRankThreads) {
+                const int x = e ^ j;
+                if (x > e) {
+                    const float u = key[e], v = key[x];
+                    if ((u > v) == ((e & k) == 0)) {
+                        key[e] = v;
+                        key[x] = u;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    int n = 0;  // distinct ones, in place: a value moves only to a lower place
+    for (int e0 = 0; e0 < cnt; e0 += kRankThreads) {
+        const int e = e0 + tid;
+        const float v = e < cnt ? key[e] : 0.0f;
+        const bool first = e < cnt && (e == 0 || !(key[e - 1] == v));
+        const unsigned b = __ballot_sync(0xffffffffu, first);
+        if (lane == 0) s_wt[warp] = __popc(b);
+        __syncthreads();
+        int off = n, tot = 0;
+        for (int w = 0; w < kRankThreads / 32; ++w) {
+            off += w < warp ? s_wt[w] : 0;
+            tot += s_wt[w];
+        }
+        off += __popc(b & ((1u << lane) - 1u));
+        if (first) {
+            key[off] = v;
+            a.thr[(size_t)f * kRankThr + off] = v;
+        }
+        n += tot;
+        __syncthreads();
+    }
+    if (tid == 0) a.n_thr[f] = n;
+    for (int k = tid; k < a.n_nodes; k += kRankThreads) {
+        const uint2 g = __ldg(nodes + k);
+        const float v = __uint_as_float(g.x);
+        if ((g.y >> 24) & 1u) {
+            if (f == 0) {
+                const uint32_t u = (uint32_t)v;
+                a.nodes[k] = make_uint2(kRankEnd | (u & 0xffu) << 11 | u >> 8, (uint32_t)k);
+            }
+        } else if ((int)((g.y >> 16) & 0xffu) == f) {
+            int lo = 0, hi = n;
+            while (lo < hi) {
+                const int mid = (lo + hi) / 2;
+                if (key[mid] < v) lo = mid + 1;
+                else hi = mid;
+            }
+            int c = 0;
+            while (c + 1 < a.n_chunks && k >= chunks[c + 1].z) ++c;
+            a.nodes[k] = make_uint2((uint32_t)(lo + 1) << 19 | (uint32_t)f << 7, (uint32_t)chunks[c].z + (g.y & 0xffffu));
+        }
+    }
+}
+
+__device__ __forceinline__ uint32_t lds32(uint32_t at) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(at));
+    return v;
+}
+
+// rf_kernel's walk over a ranked forest, which fits shared memory whole: four
+// tiles of 32 candidates per block, warp w on trees w / 4, w / 4 + 8, ... of tile
+// w mod 4.
+__global__ void __launch_bounds__(kRankWalkThreads, 2)
+rf_ranked_kernel(const __grid_constant__ RfArgs a, const uint2* __restrict__ nodes, const float* __restrict__ thr,
+                 const int32_t* __restrict__ n_thr, int n_nodes) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    uint32_t* sfeat = reinterpret_cast<uint32_t*>(smem_raw);                     // [kRankTiles][16][kRfCand] ranks plus one << 19
+    uint32_t* svote = sfeat + kRankTiles * 16 * kRfCand;                         // [kRfGroups][kRankTiles][kRfCand]
+    uint2* snodes = reinterpret_cast<uint2*>(svote + kRfGroups * kRankTiles * kRfCand);  // [n_nodes]
+    uint32_t* sroot = reinterpret_cast<uint32_t*>(snodes + n_nodes);             // [n_trees] addresses
+    const int32_t* roots = reinterpret_cast<const int32_t*>(a.forest + a.off_roots);
+    const int tid = threadIdx.x, slot = tid & (kRfCand - 1), warp = tid / 32;
+    const int half = warp % kRankTiles, grp = warp / kRankTiles;
+    const uint32_t node0 = (uint32_t)__cvta_generic_to_shared(snodes);
+    const int64_t n_work = a.list ? (int64_t)*a.n_list : a.n;
+    const int64_t n_tiles = (n_work + kRfCand - 1) / kRfCand, step_tiles = (int64_t)gridDim.x * kRankTiles;
+    const int64_t tile0 = (int64_t)blockIdx.x * kRankTiles;
+    if (tile0 < n_tiles) {
+        for (int k = tid; k < n_nodes; k += kRankWalkThreads) {
+            const uint2 g = __ldg(nodes + k);
+            snodes[k] = make_uint2(g.x, node0 + 8u * g.y);
+        }
+        for (int k = tid; k < a.n_trees; k += kRankWalkThreads) sroot[k] = node0 + 8u * (uint32_t)roots[k];
+    }
+    uint32_t feasible = 0;
+    uint32_t* feat = sfeat + half * 16 * kRfCand + slot;  // 2 KB aligned but for the slot: offsets are or-ed in
+    const uint32_t my = (uint32_t)__cvta_generic_to_shared(feat);
+    for (int64_t t0 = tile0; t0 < n_tiles; t0 += step_tiles) {
+        const int64_t pos = (t0 + half) * kRfCand + slot;
+        const bool live = pos < n_work;
+        const int64_t i = live ? (a.list ? (int64_t)a.list[pos] : pos) : 0;
+        __syncthreads();  // the previous tiles' ranks and votes are no longer read
+        for (int f = grp; f < a.d; f += kRfGroups) {
+            const uint32_t w = __ldg(a.cand + (int64_t)f * a.ld + i);
+            const float x = ((a.float_cols >> f) & 1u) ? __uint_as_float(w) : (float)(int32_t)w;
+            const float* t = thr + (size_t)f * kRankThr;
+            const int n = __ldg(n_thr + f);
+            int lo = 0;  // thresholds below x, by halving steps that are the same for every lane
+            for (int step = n > 0 ? 1 << (31 - __clz(n)) : 0; step > 0; step >>= 1)
+                if (lo + step <= n && __ldg(t + lo + step - 1) < x) lo += step;
+            feat[f * kRfCand] = x == x ? (uint32_t)(lo + 1) << 19 : kRankEnd;
+        }
+        __syncthreads();
+        uint32_t vote = 0;
+        for (int t = grp; t < a.n_trees; t += kRfGroups) {
+            uint32_t w, to;
+            auto node = [&](uint32_t at) {
+                asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(w), "=r"(to) : "r"(at));
+            };
+            auto visit = [&]() {
+                if (lds32(my + (w & 0x780u)) > w) to += 8u;
+                node(to);
+            };
+            node(sroot[t]);
+            visit();
+            visit();
+            // (bounded: a walk of the validated depth has ended by then)
+            for (int step = 2; step <= a.max_depth; step += 2) {
+                visit();
+                visit();
+                if (__all_sync(0xffffffffu, w >= kRankEnd)) break;
+            }
+            if (w < kRankEnd) atomicOr(a.err, SCOOT_DEVERR_INDEX);  // deeper than the validated depth
+            vote += (w >> 11 & 0xffu) + ((w & 0x7fu) << 8);
+        }
+        svote[(grp * kRankTiles + half) * kRfCand + slot] = vote;
+        __syncthreads();
+        if (grp == 0 && live) {
+            uint32_t v = 0;
+#pragma unroll
+            for (int g = 0; g < kRfGroups; ++g) v += svote[(g * kRankTiles + half) * kRfCand + slot];
+            a.votes[i] = v;
+            const unsigned __int128 need = (unsigned __int128)a.delta_num * a.leaf_scale * (uint32_t)a.n_trees;
+            const bool ok = (unsigned __int128)a.delta_den * v >= need;
+            if (a.mask) a.mask[i] = ok;
+            feasible += ok;
         }
     }
     if (a.count) add_count(a.count, feasible);
@@ -349,6 +560,19 @@ scoot_status scoot_rf_predict(scoot_ctx* ctx, const scoot_forest_layout* L, cons
     a.mask = mask;
     a.count = reinterpret_cast<unsigned long long*>(n_feasible);
     a.err = ctx->d_err;
+    // Ranking a forest takes a launch of 12 to 35 us.  Measured without a mask, rf_kernel
+    // against this (100 trees of 1800 nodes in all; 100 of 3300; 200 of 12100): 2^17 candidates 54 us
+    // against 52, 63 against 64, 161 against 155; 2^18 97 against 88, 112 against 107, 299 against 263;
+    // 2^20 380 against 289, 439 against 353, 1180 against 894; 2^22 4967 against 3479.
+    // With a mask about half of the pool is walked.
+    const bool ranked = L->n_nodes <= kRankNodes && L->leaf_scale <= kRankVotes &&
+                        n * L->n_trees * (L->max_depth + 1) >= (mask ? kRankFrom * 2 : kRankFrom);
+    const size_t list_bytes = mask ? ((256 + (size_t)n * 4 + 255) & ~(size_t)255) : 0;
+    const size_t node_bytes = ((size_t)L->n_nodes * 8 + 255) & ~(size_t)255;
+    if (ranked) {
+        s = scoot_workspace(ctx, list_bytes + node_bytes + (size_t)L->d * kRankThr * 4 + 256);
+        if (s != SCOOT_OK) return s;
+    }
     if (mask) {
         // Walk only the candidates still in play; the others get 0 votes.
         ScootList lst;
@@ -356,8 +580,34 @@ scoot_status scoot_rf_predict(scoot_ctx* ctx, const scoot_forest_layout* L, cons
         a.list = lst.list;
         a.n_list = lst.count;
     }
+    if (ranked) {
+        char* ws = static_cast<char*>(ctx->ws) + list_bytes;
+        RankArgs r;
+        r.forest = a.forest;
+        r.off_chunks = a.off_chunks;
+        r.off_nodes = a.off_nodes;
+        r.n_chunks = a.n_chunks;
+        r.n_nodes = L->n_nodes;
+        r.nodes = reinterpret_cast<uint2*>(ws);
+        r.thr = reinterpret_cast<float*>(ws + node_bytes);
+        r.n_thr = reinterpret_cast<int32_t*>(ws + node_bytes + (size_t)L->d * kRankThr * 4);
+        rank_forest_kernel<<<(unsigned)L->d, kRankThreads, 0, st>>>(r);
+        SCOOT_LAUNCHED(ctx);
+        const size_t rsmem = (size_t)kRankTiles * 16 * kRfCand * 4 + (size_t)kRfGroups * kRankTiles * kRfCand * 4 +
+                             (size_t)L->n_nodes * 8 + (size_t)L->n_trees * 4;
+        auto kern = rf_ranked_kernel;
+        SCOOT_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem));
+        int fit = 0;
+        SCOOT_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, kRankWalkThreads, rsmem));
+        if (fit < 1) return scoot_fail(ctx, SCOOT_EUNSUPPORTED, "forest does not fit in shared memory");
+        const int64_t grid = std::min<int64_t>((int64_t)sm_count(ctx->device) * fit,
+                                               (n + kRankTiles * kRfCand - 1) / (kRankTiles * kRfCand));
+        kern<<<(unsigned)grid, kRankWalkThreads, rsmem, st>>>(a, r.nodes, r.thr, r.n_thr, L->n_nodes);
+        SCOOT_LAUNCHED(ctx);
+        return SCOOT_OK;
+    }
     a.max_chunk_nodes = max_chunk_nodes;
-    const size_t smem = (size_t)max_chunk_nodes * 8 + (size_t)kRfCand * (L->d | 1) * 4 +
+    const size_t smem = (size_t)max_chunk_nodes * 8 + (size_t)kRfCand * L->d * 4 +
                         (size_t)kRfGroups * kRfCand * 4 + (size_t)L->n_trees * 4;
     SCOOT_CUDA(ctx, cudaFuncSetAttribute(rf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
