@@ -482,7 +482,7 @@ gp_chol_cluster_kernel(const __grid_constant__ GpPrepArgs a) {
 }
 
 constexpr int kMleMaxP = SCOOT_MAX_DIM + 2;  // ln l_1 .. ln l_d, ln s_f^2, ln tau^2
-constexpr int kSmemMleMaxN = 128;             // A and W in shared memory up to this n
+constexpr int kMleNoScratchN = 128;           // no scratch up to this n (the cluster kernel's, and more, fits)
 constexpr int kMleThreads = 512;
 
 struct MleArgs {
@@ -498,7 +498,7 @@ struct MleArgs {
     double* theta;                           // [S][M][P]
     double* lml;                             // [S][M]
     double* grad;                            // [S][M][P] or nullptr
-    double* scratch;                         // [S M][2][tri] when n > kSmemMleMaxN
+    double* scratch;                         // [S M][2][tri] when n > kMleNoScratchN
 };
 
 // Features of the observations, once per call: one thread per (j, c).
@@ -532,11 +532,12 @@ __device__ __forceinline__ void matern_slope(double r2, int kernel, double* k, d
         *dk = -1.5 * e;
     } else {
         const double a = 2.23606797749979 * r, e = exp(-a);
-        *k = (1.0 + a + a * a / 3.0) * e;
+        *k = fma(a, fma(a, 1.0 / 3.0, 1.0), 1.0) * e;
         *dk = -(5.0 / 6.0) * (1.0 + a) * e;
     }
 }
 
+// (For more observations than gp_mle_cluster_kernel holds.)
 // One block per (start s, objective m): `steps` projected Adam steps on the
 // log marginal likelihood (beta1 0.9, beta2 0.999, eps 1e-8, step size
 // lr (1 - t / steps)), then the likelihood and gradient at the result.  Each
@@ -556,15 +557,8 @@ __global__ void __launch_bounds__(kMleThreads) gp_mle_kernel(const __grid_consta
     double* al = z + n;                                  // [n] alpha
     double* col = al + n;                                // [2][n]
     double* U = col + 2 * n;                             // [d][n]: feature c of observation j at c n + j
-    double* A;
-    double* W;
-    if (n <= kSmemMleMaxN) {
-        A = U + (size_t)n * d;
-        W = A + a.tri;
-    } else {
-        A = a.scratch + (size_t)sm * 2 * a.tri;
-        W = A + a.tri;
-    }
+    double* A = a.scratch + (size_t)sm * 2 * a.tri;
+    double* W = A + a.tri;
     __shared__ double th[kMleMaxP], m1[kMleMaxP], m2[kMleMaxP], g[kMleMaxP];
     __shared__ double il2[SCOOT_MAX_DIM];  // 1 / l_c^2
     __shared__ double s_sf2, s_tau2;
@@ -710,6 +704,322 @@ __global__ void __launch_bounds__(kMleThreads) gp_mle_kernel(const __grid_consta
     if (tid == 0) a.lml[sm] = s_fail ? -INFINITY : lml;
 }
 
+// 1 / v for a normal v > 0 by Newton-Raphson from the hardware's estimate
+// (2^-20, then 2^-40, then beyond 53 bits): four dependent multiply-adds.
+__device__ __forceinline__ double rcp_newton(double v) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+    y = fma(fma(-v, y, 1.0), y, y);
+    return fma(fma(-v, y, 1.0), y, y);
+}
+
+// Whether v lies in [2^-1000, 2^1000), on the integer pipes: a pivot that
+// can be inverted (a covariance's pivots lie far inside).
+__device__ __forceinline__ bool good_pivot(double v) {
+    const int hi = __double2hiint(v);
+    return hi >= ((1023 - 1000) << 20) && hi < ((1023 + 1000) << 20);
+}
+
+// gp_mle_kernel's fit by a cluster of eight CTAs per (start, objective).
+//
+// One block per fit leaves most SMs idle at the tuning loop's 8 starts, and fp64
+// runs at two lanes per clock per SM: an evaluation at n = 128 took 1.2 ms on one
+// SM.  Here CTA r owns rows i = r (mod 8) of the symmetric matrix, and K^{-1},
+// alpha and the determinant come from one elimination: the matrix is
+// augmented by row n, which holds y^T and 0, and its first n pivots are swept,
+//   A_kk <- -1 / A_kk,  A_ik <- A_ik / A_kk,  A_ij <- A_ij - A_ik A_kj / A_kk,
+// which leaves -K^{-1}, alpha^T = y^T K^{-1} in row n and -y^T K^{-1} y at its end
+// (n^3 / 2 multiply-adds, as many as a factor, its inverse and their product;
+// the pivots are the Cholesky factor's squared).  Pivots go in blocks of eight,
+// so that a block costs one exchange: every CTA pushes its part of the next
+// block's columns into all eight CTAs' shared memory, and each inverts the
+// 8 x 8 block for itself.  The covariances and their slopes are kept for the
+// gradient where two CTAs still fit an SM (a GPU has room for 15 clusters of one
+// CTA per SM, a sixteenth would wait for them: the tuning loop has 8 starts of
+// two objectives).  An fp64 instruction holds a scheduler's unit for 64 cycles, so
+// what counts is their number: features are scaled once per evaluation,
+// categories and pivots compared as integers.
+// Measured (60 steps, 8 starts x 2 objectives, gp_mle_kernel against this): n = 64
+// 19.7 ms against 5.8, n = 128 72.8 against 17.6, n = 256 499 against 90; 64 fits at
+// n = 128 75.6 against 34.0, 128 fits 75.6 against 67.1.  Larger n than fits (about
+// 300) stay with gp_mle_kernel.  Keeping the squared differences as well cost the
+// second CTA per SM and was slower (25 ms at n = 128).
+constexpr int kMleB = kClusterCTAs;  // pivots per block: one row of a block per CTA
+constexpr int kMleClThreads = 256;
+
+constexpr size_t kMleClTwo = 108 * 1024;  // shared memory of which two CTAs fit an SM
+
+struct MleClSizes {
+    int64_t own;                  // entries of the CTA with the most
+    size_t bytes, keep_bytes;     // without and of the kept covariances
+};
+
+inline MleClSizes mle_cl_sizes(int n, int d) {
+    MleClSizes z;
+    z.own = 0;
+    for (int r = 0; r < kClusterCTAs; ++r) {
+        const int64_t nl = (n + 1 - r + kClusterCTAs - 1) / kClusterCTAs;  // rows r, r + 8, ... up to n
+        const int64_t e = nl * (r + 1) + (int64_t)kClusterCTAs * nl * (nl - 1) / 2;
+        if (e > z.own) z.own = e;
+    }
+    const size_t rows = (size_t)(n + 1 + kClusterCTAs - 1) / kClusterCTAs;
+    z.bytes = ((size_t)2 * (n + 1) * kMleB + (size_t)n * d + (size_t)z.own + 2 * (size_t)(n + 1) + rows * kMleB) * sizeof(double);
+    z.keep_bytes = 2 * (size_t)z.own * sizeof(double);
+    return z;
+}
+
+__global__ void __cluster_dims__(kClusterCTAs, 1, 1) __launch_bounds__(kMleClThreads, 2)
+gp_mle_cluster_kernel(const __grid_constant__ MleArgs a, int64_t own, int keep) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int C = kClusterCTAs, B = kMleB;
+    const int n = a.n, d = a.d, P = a.P;
+    const int rank = (int)cluster.block_rank(), sm = blockIdx.x / C, m = sm % a.M;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int nwarps = kMleClThreads / 32;
+    double* panel = reinterpret_cast<double*>(smem_raw);  // [2][n + 1][B] the pivot block's columns
+    double* U = panel + 2 * (size_t)(n + 1) * B;          // [d][n] features, ordinal ones over their lengthscale
+    double* A = U + (size_t)n * d;                        // owned rows, packed
+    double* al = A + own;                                 // [n + 1] alpha, then y^T K^{-1} y
+    double* piv = al + n + 1;                             // [n + 1]
+    double* gs = piv + n + 1;                             // [owned rows][B] a row's multipliers in an elimination step
+    double* kvs = gs + (size_t)((n + 1 + C - 1) / C) * B;  // if kept: k / s_f^2 of the owned rows
+    double* dks = kvs + own;                              // and its slope in r^2
+    __shared__ double th[kMleMaxP], g[kMleMaxP], il2[SCOOT_MAX_DIM], il[SCOOT_MAX_DIM];
+    __shared__ double s_sf2, s_tau2, s_c1, s_c2, s_total;
+    __shared__ double part[C][kMleMaxP + 1], red[nwarps][kMleMaxP + 1];
+    __shared__ double Dn[B][B + 1], rowb[2][B], rcp[2];
+    __shared__ int s_fail;
+    const int nl = (n + 1 - rank + C - 1) / C;  // owned rows, row n among them
+    double m1 = 0.0, m2 = 0.0;  // thread p: Adam's moments of parameter p
+    if (tid < P) th[tid] = a.theta0[(int64_t)sm * P + tid];
+    if (tid == 0) s_fail = 0;
+    // Term c of r^2 between rows i and k.
+    auto term = [&](int c, int i, int k) {
+        const double x = U[c * n + i], y = U[c * n + k];
+        if ((a.cat_mask >> c) & 1u) return __double_as_longlong(x) != __double_as_longlong(y) ? il2[c] : 0.0;
+        return (x - y) * (x - y);
+    };
+    auto distance2 = [&](int i, int k) {
+        double r2 = 0.0;
+        for (int c = 0; c < d; ++c) {
+            const double x = U[c * n + i], y = U[c * n + k];
+            if ((a.cat_mask >> c) & 1u) {
+                if (__double_as_longlong(x) != __double_as_longlong(y)) r2 += il2[c];
+            } else {
+                r2 = fma(x - y, x - y, r2);
+            }
+        }
+        return r2;
+    };
+    double* peer[C];  // every CTA's panel
+#pragma unroll
+    for (int r = 0; r < C; ++r) peer[r] = cluster.map_shared_rank(panel, r);
+    // The columns kb .. kb + 7 of the symmetric matrix into every CTA's panel,
+    // [j][c] = A_j,kb+c (0 beyond the last pivot): an owned row j >= kb + c gives
+    // its entries, the block's own rows those of the rows before them.
+    auto push = [&](int kb) {
+        const size_t off = (size_t)((kb / B) & 1) * (n + 1) * B;
+        for (int e = tid; e < nl * B; e += kMleClThreads) {
+            const int li = e / B, c = e - li * B, i = rank + C * li, kc = kb + c;
+            if (kc < n && kc > i) continue;
+            const double v = kc < n ? A[local_row_off(li, rank) + kc] : 0.0;
+#pragma unroll
+            for (int r = 0; r < C; ++r) peer[r][off + i * B + c] = v;
+        }
+        const int row = kb + rank;
+        if (row < n) {
+            const double* Ar = A + local_row_off(row / C, rank);
+            for (int j = tid; j < row; j += kMleClThreads) {
+                const double v = Ar[j];
+#pragma unroll
+                for (int r = 0; r < C; ++r) peer[r][off + j * B + rank] = v;
+            }
+        }
+    };
+    double lml = 0.0;
+    for (int it = 0; it <= a.steps; ++it) {
+        __syncthreads();
+        if (tid < d) {
+            il[tid] = exp(-th[tid]);
+            il2[tid] = il[tid] * il[tid];
+        } else if (tid == 32) s_sf2 = exp(th[d]);
+        else if (tid == 64) s_tau2 = exp(th[d + 1]);
+        else if (tid == 96) s_c1 = 1.0 - pow(0.9, it + 1);
+        else if (tid == 128) s_c2 = 1.0 - pow(0.999, it + 1);
+        __syncthreads();
+        const double sf2 = s_sf2, tau2 = s_tau2;
+        for (int t = tid; t < n * d; t += kMleClThreads) {
+            const int c = t % d;
+            const double u = a.U[t];
+            U[c * n + t / d] = ((a.cat_mask >> c) & 1u) ? u : u * il[c];
+        }
+        __syncthreads();
+        for (int li = warp; li < nl; li += nwarps) {
+            const int i = rank + C * li;
+            const int64_t o = local_row_off(li, rank);
+            if (i == n) {
+                for (int k = lane; k <= n; k += 32) A[o + k] = k < n ? (double)a.y[(int64_t)m * n + k] : 0.0;
+                continue;
+            }
+            for (int k = lane; k <= i; k += 32) {
+                double kv, dk;
+                matern_slope(distance2(i, k), a.kernel, &kv, &dk);
+                if (keep) {
+                    kvs[o + k] = kv;
+                    dks[o + k] = dk;
+                }
+                A[o + k] = sf2 * kv + (i == k ? tau2 : 0.0);
+            }
+        }
+        __syncthreads();
+        push(0);
+        cluster.sync();
+        for (int kb = 0; kb < n; kb += B) {
+            const double* P0 = panel + (size_t)((kb / B) & 1) * (n + 1) * B;
+            const int be = min(B, n - kb);
+            if (warp < 2) {  // minus the inverse of the pivot block, an entry per thread
+                const int r = tid / B, c = tid % B;
+                double e = r < be && c < be ? P0[(kb + r) * B + c] : 0.0;
+                for (int p = 0; p < be; ++p) {
+                    if (r == p) rowb[p & 1][c] = e;
+                    asm volatile("bar.sync 1, 64;" ::: "memory");
+                    const double x = rowb[p & 1][r], y = rowb[p & 1][c];
+                    if (r == p && c == p) {  // (while the others multiply)
+                        piv[kb + p] = e;
+                        const bool ok = good_pivot(e);
+                        if (!ok) s_fail = 1;
+                        rcp[p & 1] = ok ? rcp_newton(e) : 0.0;
+                    }
+                    const double xy = r == p ? y : c == p ? x : -x * y;
+                    asm volatile("bar.sync 1, 64;" ::: "memory");
+                    const double q = rcp[p & 1];
+                    e = r == p ? (c == p ? -q : xy * q) : (c == p ? xy * q : fma(xy, q, e));
+                }
+                Dn[r][c] = r < be && c < be ? e : 0.0;
+            }
+            __syncthreads();
+            if (s_fail) break;  // the same in every CTA: each has swept the same block
+            for (int e = tid; e < nl * B; e += kMleClThreads) {  // the rows' multipliers
+                const int li = e / B, c = e - li * B, i = rank + C * li, ii = i - kb;
+                double v = 0.0;
+                if (ii >= 0 && ii < be) {
+                    v = -Dn[c][ii];
+                } else {
+#pragma unroll
+                    for (int p = 0; p < B; ++p) v = fma(P0[i * B + p], -Dn[p][c], v);
+                }
+                gs[e] = v;
+            }
+            __syncthreads();
+            for (int li = warp; li < nl; li += nwarps) {
+                const int i = rank + C * li, ii = i - kb;
+                const bool pivot = ii >= 0 && ii < be;
+                double* Ai = A + local_row_off(li, rank);
+                double gr[B];
+#pragma unroll
+                for (int c = 0; c < B; ++c) gr[c] = gs[li * B + c];
+                for (int j = lane; j <= i; j += 32) {
+                    const int jj = j - kb;
+                    if (jj >= 0 && jj < be) {
+                        Ai[j] = pivot ? Dn[ii][jj] : gs[li * B + jj];
+                    } else {
+                        const double* Pj = P0 + (size_t)j * B;
+                        double v = pivot ? 0.0 : -Ai[j];
+#pragma unroll
+                        for (int c = 0; c < B; ++c) v = fma(gr[c], Pj[c], v);
+                        Ai[j] = pivot ? v : -v;
+                    }
+                }
+            }
+            __syncthreads();
+            if (kb + B < n) {
+                push(kb + B);
+            } else if (n % C == rank) {  // row n: alpha and -y^T alpha, everywhere
+                const double* Ar = A + local_row_off(n / C, rank);
+                for (int j = tid; j <= n; j += kMleClThreads)
+                    for (int r = 0; r < C; ++r) cluster.map_shared_rank(al, r)[j] = j < n ? Ar[j] : -Ar[j];
+            }
+            cluster.sync();
+        }
+        if (s_fail) break;
+        double acc[kMleMaxP + 1];
+#pragma unroll
+        for (int p = 0; p <= kMleMaxP; ++p) acc[p] = 0.0;
+        for (int li = warp; li < nl; li += nwarps) {
+            const int i = rank + C * li;
+            if (i == n) continue;
+            const int64_t o = local_row_off(li, rank);
+            const double ai = al[i];
+            for (int k = lane; k <= i; k += 32) {
+                const double w = fma(ai, al[k], A[o + k]) * (i == k ? 0.5 : 1.0);  // A holds -K^{-1}
+                if (i == k) {
+                    acc[kMleMaxP - 1] += w * tau2;
+                    acc[kMleMaxP - 2] += w * sf2;  // k(0) = 1
+                    continue;
+                }
+                double kv, dk;
+                if (keep) {
+                    kv = kvs[o + k];
+                    dk = dks[o + k];
+                } else {
+                    matern_slope(distance2(i, k), a.kernel, &kv, &dk);
+                }
+                const double f = -2.0 * sf2 * dk * w;
+#pragma unroll
+                for (int c = 0; c < SCOOT_MAX_DIM; ++c)
+                    if (c < d) acc[c] = fma(f, term(c, i, k), acc[c]);
+                acc[kMleMaxP - 2] = fma(w * sf2, kv, acc[kMleMaxP - 2]);
+            }
+        }
+        if (it == a.steps && rank == 0)  // the likelihood, at the result alone
+            for (int p = tid; p < n; p += kMleClThreads) acc[kMleMaxP] += log(piv[p]);
+#pragma unroll
+        for (int p = 0; p <= kMleMaxP; ++p) {
+            if (p < d || p >= kMleMaxP - 2) {
+                double v = acc[p];
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (lane == 0) red[warp][p] = v;
+            }
+        }
+        __syncthreads();
+        if (tid < d || (tid >= kMleMaxP - 2 && tid <= kMleMaxP)) {
+            double v = 0.0;
+            for (int w2 = 0; w2 < nwarps; ++w2) v += red[w2][tid];
+            for (int r = 0; r < C; ++r) cluster.map_shared_rank(&part[0][0], r)[rank * (kMleMaxP + 1) + tid] = v;
+        }
+        cluster.sync();
+        if (tid < d || (tid >= kMleMaxP - 2 && tid <= kMleMaxP)) {
+            double v = 0.0;
+            for (int r = 0; r < C; ++r) v += part[r][tid];
+            if (tid < d) g[tid] = v;
+            else if (tid == kMleMaxP) s_total = v;
+            else g[tid - (kMleMaxP - 2) + d] = v;
+        }
+        __syncthreads();
+        if (it == a.steps) {
+            lml = -0.5 * (al[n] + s_total) - 0.5 * n * 1.8378770664093453;  // log(2 pi)
+            break;
+        }
+        if (tid < P && ((a.free_mask >> tid) & 1u)) {  // projected Adam step on the free parameters
+            const double step = a.lr * (1.0 - (double)it / a.steps), gp = g[tid];
+            m1 = 0.9 * m1 + 0.1 * gp;
+            m2 = 0.999 * m2 + 0.001 * gp * gp;
+            const double upd = step * (m1 / s_c1) / (sqrt(m2 / s_c2) + 1e-8);
+            th[tid] = fmin(fmax(th[tid] + upd, a.lo[tid]), a.hi[tid]);
+        }
+    }
+    if (rank == 0) {
+        if (tid < P) {
+            a.theta[(int64_t)sm * P + tid] = th[tid];
+            if (a.grad) a.grad[(int64_t)sm * P + tid] = s_fail ? 0.0 : g[tid];
+        }
+        if (tid == 0) a.lml[sm] = s_fail ? -INFINITY : lml;
+    }
+    cluster.sync();  // no CTA leaves while another may still write to it
+}
+
 }  // namespace
 
 extern "C" {
@@ -846,7 +1156,7 @@ scoot_status scoot_gp_mle_work_bytes(int32_t n, int32_t d, int32_t n_obj, int32_
     if (!bytes || n < 1 || d < 1 || n_obj < 1 || n_starts < 1) return SCOOT_EINVAL;
     const int64_t tri = (int64_t)n * (n + 1) / 2;
     int64_t b = ((int64_t)n * d * 8 + 255) / 256 * 256;
-    if (n > kSmemMleMaxN) b += (int64_t)n_starts * n_obj * 2 * tri * 8;
+    if (n > kMleNoScratchN) b += (int64_t)n_starts * n_obj * 2 * tri * 8;
     *bytes = b;
     return SCOOT_OK;
 }
@@ -925,12 +1235,23 @@ scoot_status scoot_gp_mle(scoot_ctx* ctx, const scoot_param* h_space, int32_t d,
     a.theta = theta;
     a.lml = lml;
     a.grad = grad;
-    a.scratch = n > kSmemMleMaxN ? reinterpret_cast<double*>(ws + ((int64_t)n * d * 8 + 255) / 256 * 256) : nullptr;
+    a.scratch = n > kMleNoScratchN ? reinterpret_cast<double*>(ws + ((int64_t)n * d * 8 + 255) / 256 * 256) : nullptr;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     mle_feat_kernel<<<(n * d + kFeatThreads - 1) / kFeatThreads, kFeatThreads, 0, st>>>(f);
     SCOOT_LAUNCHED(ctx);
-    const size_t smem = (size_t)(7 * n + (size_t)n * d) * sizeof(double) +
-                        (n <= kSmemMleMaxN ? (size_t)2 * a.tri * sizeof(double) : 0);
+    int optin = 0;
+    SCOOT_CUDA(ctx, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
+    const MleClSizes cl = mle_cl_sizes(n, d);
+    if (cl.bytes + 8192 <= (size_t)optin) {
+        const int keep = cl.bytes + cl.keep_bytes <= kMleClTwo || (cl.bytes > kMleClTwo && cl.bytes + cl.keep_bytes + 8192 <= (size_t)optin);
+        const size_t bytes = cl.bytes + (keep ? cl.keep_bytes : 0);
+        SCOOT_CUDA(ctx, cudaFuncSetAttribute(gp_mle_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+        gp_mle_cluster_kernel<<<n_starts * n_obj * kClusterCTAs, kMleClThreads, bytes, st>>>(a, cl.own, keep);
+        SCOOT_LAUNCHED(ctx);
+        return SCOOT_OK;
+    }
+    if (!a.scratch) return scoot_fail(ctx, SCOOT_EUNSUPPORTED, "shared memory of %d bytes is too small", optin);
+    const size_t smem = (size_t)(7 * n + (size_t)n * d) * sizeof(double);
     SCOOT_CUDA(ctx, cudaFuncSetAttribute(gp_mle_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     gp_mle_kernel<<<n_starts * n_obj, kMleThreads, smem, st>>>(a);
     SCOOT_LAUNCHED(ctx);
