@@ -26,7 +26,7 @@ constexpr int kKmatThreads = 128;
 constexpr int kCholThreads = 1024;
 constexpr int kRowBlockDev = 64;   // rows of L^{-1} per tile (the layout's)
 constexpr int kColChunkDev = 32;   // columns of L^{-1} per tile
-constexpr int kSmemCholMaxN = 160; // A and W (packed lower triangles, fp64) in shared memory up to this n
+constexpr int kOneTriangleN = 160; // scratch of one packed triangle per objective up to this n, of two above
 
 struct GpPrepArgs {
     int32_t n, d, M, kernel, n_ord, n_pat, n_rb, n_tiles;
@@ -47,7 +47,7 @@ struct GpPrepArgs {
     int64_t off_fmap, off_xs, off_ils, off_alpha, off_linv, off_scal, off_cat, off_warp;
     double* U;                          // [M][n][d] scaled features, source order
     double* K;                          // [M][tri] packed lower triangle of K + tau^2 I (factorised in place when n is large)
-    double* W;                          // [M][tri] elimination of the identity (n large)
+    double* W;                          // [M][tri] elimination of the identity (NULL up to kOneTriangleN)
     uint32_t* err;
 };
 
@@ -253,6 +253,7 @@ __device__ bool eliminate(double* A, double* W, double* col, double* rinv, doubl
     return ok;
 }
 
+// (For more observations than gp_chol_cluster_kernel holds.)
 // One block per objective: the factorisation with L^{-1} alongside, then
 // alpha, the best observed y and the fp32 tiles of L^{-1}.
 __global__ void __launch_bounds__(kCholThreads) gp_chol_kernel(const __grid_constant__ GpPrepArgs a) {
@@ -263,16 +264,8 @@ __global__ void __launch_bounds__(kCholThreads) gp_chol_kernel(const __grid_cons
     double* rinv2 = rinv + n;                            // [n] 1 / pivot^2
     double* z = rinv2 + n;                               // [n] L^{-1} y
     double* col = z + n;                                 // [2][n] column j of A
-    double* A;
-    double* W;
-    if (n <= kSmemCholMaxN) {
-        A = col + 2 * n;
-        W = A + a.tri;
-        for (int64_t t = tid; t < a.tri; t += kCholThreads) A[t] = a.K[(int64_t)m * a.tri + t];
-    } else {
-        A = a.K + (int64_t)m * a.tri;
-        W = a.W + (int64_t)m * a.tri;
-    }
+    double* A = a.K + (int64_t)m * a.tri;
+    double* W = a.W + (int64_t)m * a.tri;
     if (!eliminate(A, W, col, rinv, rinv2, n)) {
         if (tid == 0) atomicOr(a.err, SCOOT_DEVERR_VALUE);
         return;
@@ -318,7 +311,7 @@ __global__ void __launch_bounds__(kCholThreads) gp_chol_kernel(const __grid_cons
 
 constexpr int kClusterCTAs = 8;          // CTAs sharing one factorisation (portable cluster size)
 constexpr int kClusterThreads = 256;
-constexpr int kClusterMaxN = 384;        // rows of A and W split over the cluster's shared memory
+constexpr int kClusterB = kClusterCTAs;  // pivots per block: one row of a block per CTA
 
 // Offset of local row li (global row rank + C li) in a CTA's packed rows:
 // row i holds i + 1 entries.
@@ -326,159 +319,212 @@ __device__ __forceinline__ int64_t local_row_off(int li, int rank) {
     return (int64_t)li * (rank + 1) + (int64_t)kClusterCTAs * li * (li - 1) / 2;
 }
 
-// The factorisation of gp_chol_kernel spread over a cluster of kClusterCTAs
-// CTAs (one cluster per objective): CTA r owns rows i = r (mod C) of A and
-// W in its shared memory.  What a step needs from other rows travels through
-// distributed shared memory before the step's cluster barrier: the thread
-// that finishes A_i,j+1 stores it into every CTA's copy of the next pivot
-// column, the row j+1 of W is stored the same way as its entries become
-// final, and the thread that finishes the next diagonal entry stores its
-// reciprocals (or the failure) everywhere.  Then z = L^{-1} y per owned row
-// (broadcast), per-CTA partial sums of alpha = L^{-T} z over owned rows
-// (added in rank order by CTA 0), and each CTA writes its rows' tiles.
+// Entries of the CTA with the most, of rows 0 .. n over a cluster.
+inline int64_t cluster_own(int n) {
+    int64_t own = 0;
+    for (int r = 0; r < kClusterCTAs; ++r) {
+        const int64_t nl = (n + 1 - r + kClusterCTAs - 1) / kClusterCTAs;
+        const int64_t e = nl * (r + 1) + (int64_t)kClusterCTAs * nl * (nl - 1) / 2;  // local_row_off(nl, r)
+        if (e > own) own = e;
+    }
+    return own;
+}
+
+// 1 / v for a normal v > 0 by Newton-Raphson from the hardware's estimate
+// (2^-20, then 2^-40, then beyond 53 bits): four dependent multiply-adds.
+__device__ __forceinline__ double rcp_newton(double v) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+    y = fma(fma(-v, y, 1.0), y, y);
+    return fma(fma(-v, y, 1.0), y, y);
+}
+
+// Whether v lies in [2^-1000, 2^1000), on the integer pipes: a pivot that
+// can be inverted (a covariance's pivots lie far inside).
+__device__ __forceinline__ bool good_pivot(double v) {
+    const int hi = __double2hiint(v);
+    return hi >= ((1023 - 1000) << 20) && hi < ((1023 + 1000) << 20);
+}
+
+// Bytes of shared memory of gp_chol_cluster_kernel.
+inline size_t chol_cluster_bytes(int n) {
+    const size_t rows = (size_t)(n + 1 + kClusterCTAs - 1) / kClusterCTAs;
+    return ((size_t)cluster_own(n) + 2 * (size_t)(n + 1) * kClusterB + rows * kClusterB) * sizeof(double);
+}
+
+// gp_chol_kernel's results by a cluster of eight CTAs per objective, in blocks of
+// eight pivots.  CTA r owns rows i = r (mod 8) of K + tau^2 I, augmented by row n,
+// which holds y^T.  The elimination is in place: entry t of row i holds A_it
+// before pivot t and W_it, the elimination of the identity, after it.  A block of
+// pivots kb .. kb + 7 with D = A_kb..kb+7 = L_D L_D^T (X = L_D^{-1}) finishes its
+// rows of L^{-1}, X W, and takes from every later row i
+//   A_ij -= g_i . A_j,block,   W_it -= g_i . W_block,t,   g_i = A_i,block D^{-1}
+// so that row n ends as -alpha^T = -y^T (K + tau^2 I)^{-1}.  What a block needs of
+// other CTAs' rows is one panel of eight values per row or column, which every
+// CTA pushes its part of into all eight CTAs' shared memory: one cluster barrier
+// per eight pivots (one per pivot and two triangles before).  Each CTA
+// factorises the 8 x 8 block for itself.
+// Bound by the chain of pivots and the fp64 units (64 cycles a warp instruction
+// and scheduler).  n = 200, three objectives: 288 us, 560 with a barrier per pivot.
 __global__ void __cluster_dims__(kClusterCTAs, 1, 1) __launch_bounds__(kClusterThreads)
-gp_chol_cluster_kernel(const __grid_constant__ GpPrepArgs a) {
+gp_chol_cluster_kernel(const __grid_constant__ GpPrepArgs a, int64_t own) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int n = a.n, C = kClusterCTAs;
-    const int rank = (int)cluster.block_rank(), m = blockIdx.x / C;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = kClusterThreads / 32;
-    double* rinv = reinterpret_cast<double*>(smem_raw);  // [n]
-    double* rinv2 = rinv + n;                            // [n]
-    double* col = rinv2 + n;                             // [2][n] pivot column
-    double* wrow = col + 2 * n;                          // [2][n] row j of W
-    double* z = wrow + 2 * n;                            // [n]
-    double* part = z + n;                                // [n] this CTA's share of alpha
-    const int nl = (n - rank + C - 1) / C;               // rows owned
-    double* A = part + n;                                // owned rows, packed
-    double* W = A + local_row_off(nl, rank);
-    __shared__ int s_bad_at;
+    constexpr int C = kClusterCTAs, B = kClusterB, nwarps = kClusterThreads / 32;
+    const int n = a.n, rank = (int)cluster.block_rank(), m = blockIdx.x / C;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double* panel = reinterpret_cast<double*>(smem_raw);  // [2][n + 1][B]
+    double* A = panel + 2 * (size_t)(n + 1) * B;          // owned rows, packed
+    double* gs = A + own;                                 // [owned rows][B] the rows' g
+    const int nl = (n + 1 - rank + C - 1) / C;            // rows owned, row n among them
+    __shared__ double Di[B][B + 1], X[B][B + 1], Xq[B][B + 1], rowa[2][B], roww[2][B], rcp[B], rs[B];
+    __shared__ int s_fail;
     const double* K = a.K + (int64_t)m * a.tri;
-    // load owned rows; W = I
-    for (int li = warp; li < nl; li += nwarps) {
-        const int i = rank + C * li;
-        const int64_t o = local_row_off(li, rank);
-        for (int t = lane; t <= i; t += 32) {
-            A[o + t] = K[tri_idx(i, t)];
-            W[o + t] = t == i ? 1.0 : 0.0;
-        }
-    }
-    // the first pivot column, row 0 of W and the first pivot, everywhere
-    for (int li = tid; li < nl; li += kClusterThreads) {
-        const int i = rank + C * li;
-        const double v = K[tri_idx(i, 0)];
-        for (int r = 0; r < C; ++r) cluster.map_shared_rank(col, r)[i] = v;
-    }
-    if (tid == 0) {
-        const double s0 = K[0];
-        const bool bad = !(s0 > 0.0) || !isfinite(s0);
-        s_bad_at = bad ? 0 : n;
-        rinv[0] = bad ? 0.0 : rsqrt_newton(s0);
-        rinv2[0] = rinv[0] * rinv[0];
-        wrow[0] = 1.0;
-    }
-    cluster.sync();
-    for (int j = 0; j < n; ++j) {
-        if (s_bad_at <= j) break;  // the same in every thread of the cluster
-        const double r2 = rinv2[j];
-        const double* cj = col + (j & 1) * n;
-        const double* wj = wrow + (j & 1) * n;
-        const int nb = (j + 1) & 1;
-        // owned rows i > j
-        int li0 = (j + 1 - rank + C - 1) / C;
-        if (li0 < 0) li0 = 0;
-        for (int li = li0 + warp; li < nl; li += nwarps) {
-            const int i = rank + C * li;
-            const int64_t o = local_row_off(li, rank);
-            const double g = cj[i] * r2;
-            for (int t = lane; t <= i; t += 32) {
-                double* dst = t <= j ? W + o + t : A + o + t;
-                const double src = t <= j ? wj[t] : cj[t];
-                const double v = *dst - g * src;
-                *dst = v;
-                if (t == j + 1) {  // A_i,j+1 is final: the next pivot column, everywhere
-                    for (int r = 0; r < C; ++r) cluster.map_shared_rank(col + nb * n, r)[i] = v;
-                    if (i == j + 1) {
-                        if (!(v > 0.0) || !isfinite(v)) {
-                            for (int r = 0; r < C; ++r) *cluster.map_shared_rank(&s_bad_at, r) = j + 1;
-                        } else {
-                            const double y = rsqrt_newton(v);
-                            for (int r = 0; r < C; ++r) {
-                                cluster.map_shared_rank(rinv, r)[j + 1] = y;
-                                cluster.map_shared_rank(rinv2, r)[j + 1] = y * y;
-                            }
-                        }
-                    }
-                }
-                if (i == j + 1 && t <= j)  // W_j+1,t is final: row j + 1 of W, everywhere
-                    for (int r = 0; r < C; ++r) cluster.map_shared_rank(wrow + nb * n, r)[t] = v;
-            }
-            if (i == j + 1 && lane == 0)
-                for (int r = 0; r < C; ++r) cluster.map_shared_rank(wrow + nb * n, r)[j + 1] = 1.0;
-        }
-        cluster.sync();
-    }
-    if (s_bad_at < n) {  // the same everywhere; no shared memory of another CTA is touched after this
-        if (tid == 0 && rank == 0) atomicOr(a.err, SCOOT_DEVERR_VALUE);
-        return;
-    }
     const float* y = a.y + (int64_t)m * n;
-    // z_i for owned rows, everywhere
+    if (tid == 0) s_fail = 0;
     for (int li = warp; li < nl; li += nwarps) {
         const int i = rank + C * li;
-        const int64_t o = local_row_off(li, rank);
-        double t = 0.0;
-        for (int c = lane; c <= i; c += 32) t += W[o + c] * (double)y[c];
-        for (int sh = 16; sh > 0; sh >>= 1) t += __shfl_xor_sync(0xffffffffu, t, sh);
-        if (lane == 0) {
-            const double zi = t * rinv[i];
-            for (int r = 0; r < C; ++r) cluster.map_shared_rank(z, r)[i] = zi;
+        double* Ai = A + local_row_off(li, rank);
+        for (int t = lane; t <= i; t += 32) Ai[t] = i < n ? K[tri_idx(i, t)] : t < n ? (double)y[t] : 0.0;
+    }
+    double* peer[C];  // every CTA's panel
+#pragma unroll
+    for (int r = 0; r < C; ++r) peer[r] = cluster.map_shared_rank(panel, r);
+    // The panel of block kb: [j][c] = A_j,kb+c of the rows j >= kb + c (and its
+    // mirror within the block), W_kb+c,j of the columns j < kb; 0 beyond pivot n - 1.
+    auto push = [&](int kb) {
+        const size_t off = (size_t)((kb / B) & 1) * (n + 1) * B;
+        for (int e = tid; e < nl * B; e += kClusterThreads) {
+            const int li = e / B, c = e - li * B, i = rank + C * li, kc = kb + c;
+            if (kc < n && (i < kb || kc > i)) continue;
+            const double v = kc < n ? A[local_row_off(li, rank) + kc] : 0.0;
+#pragma unroll
+            for (int r = 0; r < C; ++r) peer[r][off + i * B + c] = v;
+        }
+        const int row = kb + rank;
+        if (row < n) {
+            const double* Ar = A + local_row_off(row / C, rank);
+            for (int j = tid; j < row; j += kClusterThreads) {
+                const double v = Ar[j];
+#pragma unroll
+                for (int r = 0; r < C; ++r) peer[r][off + j * B + rank] = v;
+            }
+        }
+    };
+    __syncthreads();
+    push(0);
+    cluster.sync();
+    for (int kb = 0; kb < n; kb += B) {
+        const double* P0 = panel + (size_t)((kb / B) & 1) * (n + 1) * B;
+        const int be = min(B, n - kb);
+        if (warp < 2) {  // X and D^{-1}, an entry per thread
+            const int r = tid / B, c = tid % B;
+            double e = r < be && c < be ? P0[(kb + r) * B + c] : 0.0, w = r == c && r < be ? 1.0 : 0.0;
+            for (int p = 0; p < be; ++p) {
+                if (r == p) {
+                    rowa[p & 1][c] = e;
+                    roww[p & 1][c] = w;
+                }
+                asm volatile("bar.sync 1, 64;" ::: "memory");
+                if (r == p && c == p) {  // (while the others multiply)
+                    const bool ok = good_pivot(e);
+                    if (!ok) s_fail = 1;
+                    rcp[p] = ok ? rcp_newton(e) : 0.0;
+                }
+                const double x = r > p ? -rowa[p & 1][r] : 0.0, xa = x * rowa[p & 1][c], xw = x * roww[p & 1][c];
+                asm volatile("bar.sync 1, 64;" ::: "memory");
+                e = fma(xa, rcp[p], e);
+                w = fma(xw, rcp[p], w);
+            }
+            X[r][c] = w;  // of unit diagonal: row r of L_D^{-1} is this over sqrt(pivot r)
+            Xq[r][c] = r < be ? w * rcp[r] : 0.0;
+            asm volatile("bar.sync 1, 64;" ::: "memory");
+            double v = 0.0;
+            for (int p = 0; p < be; ++p) v = fma(Xq[p][r], X[p][c], v);
+            Di[r][c] = v;
+        }
+        __syncthreads();
+        if (s_fail) break;  // the same in every CTA: each has factorised the same block
+        if (tid >= kClusterThreads - be) {  // 1 / sqrt(pivot), for the block's rows
+            const double q = rcp[tid - (kClusterThreads - be)];
+            rs[tid - (kClusterThreads - be)] = q * rsqrt_newton(q);
+        }
+        for (int e = tid; e < nl * B; e += kClusterThreads) {  // g of the later rows
+            const int li = e / B, c = e - li * B, i = rank + C * li;
+            double v = 0.0;
+            if (i >= kb + be) {
+#pragma unroll
+                for (int p = 0; p < B; ++p) v = fma(P0[i * B + p], Di[p][c], v);
+            }
+            gs[e] = v;
+        }
+        __syncthreads();
+        for (int li = (kb / C) + warp; li < nl; li += nwarps) {
+            const int i = rank + C * li, ii = i - kb;
+            if (ii < 0) continue;
+            double* Ai = A + local_row_off(li, rank);
+            if (ii < be) {  // a row of the block: L^{-1} of it
+                const double s = rs[ii];
+                for (int t = lane; t <= i; t += 32) {
+                    double v = 0.0;
+                    if (t < kb) {
+                        for (int p = 0; p <= ii; ++p) v = fma(X[ii][p], P0[(size_t)t * B + p], v);
+                    } else {
+                        v = X[ii][t - kb];
+                    }
+                    Ai[t] = v * s;
+                }
+                continue;
+            }
+            double gr[B];
+#pragma unroll
+            for (int c = 0; c < B; ++c) gr[c] = -gs[li * B + c];
+            for (int j = lane; j <= i; j += 32) {
+                const int jj = j - kb;
+                if (jj >= 0 && jj < be) {
+                    Ai[j] = -gs[li * B + jj];
+                } else {
+                    const double* Pj = P0 + (size_t)j * B;
+                    double v = Ai[j];
+#pragma unroll
+                    for (int c = 0; c < B; ++c) v = fma(gr[c], Pj[c], v);
+                    Ai[j] = v;
+                }
+            }
+        }
+        __syncthreads();
+        if (kb + B < n) {
+            push(kb + B);
+            cluster.sync();
         }
     }
-    cluster.sync();
-    // this CTA's share of alpha_c = sum over owned rows i >= c of L^{-1}_ic z_i
-    for (int c = tid; c < n; c += kClusterThreads) {
-        double t = 0.0;
-        int li = (c - rank + C - 1) / C;
-        if (li < 0) li = 0;
-        for (; li < nl; ++li) {
-            const int i = rank + C * li;
-            t += W[local_row_off(li, rank) + c] * rinv[i] * z[i];
+    if (s_fail) {  // the same everywhere
+        if (tid == 0 && rank == 0) atomicOr(a.err, SCOOT_DEVERR_VALUE);
+    } else {
+        if (n % C == rank) {  // row n: minus alpha
+            const double* Ar = A + local_row_off(n / C, rank);
+            float* alpha = reinterpret_cast<float*>(a.blob + a.off_alpha) + (int64_t)m * n;
+            for (int c = tid; c < n; c += kClusterThreads) alpha[c] = (float)-Ar[c];
         }
-        part[c] = t;
-    }
-    cluster.sync();
-    if (rank == 0) {
-        float* alpha = reinterpret_cast<float*>(a.blob + a.off_alpha) + (int64_t)m * n;
-        for (int c = tid; c < n; c += kClusterThreads) {
-            double t = 0.0;
-            for (int r = 0; r < C; ++r) t += cluster.map_shared_rank(part, r)[c];
-            alpha[c] = (float)t;
-        }
-        if (warp == 0) {
+        if (rank == 0 && warp == 0) {
             float best = -INFINITY;
             for (int j = lane; j < n; j += 32) best = fmaxf(best, y[j]);
             for (int sh = 16; sh > 0; sh >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, sh));
             if (lane == 0) reinterpret_cast<float*>(a.blob + a.off_scal)[m * 4 + 2] = best;
         }
+        // tiles: the owner of a row writes its entries and zeros (CTA 0 the padding rows)
+        float* tiles = reinterpret_cast<float*>(a.blob + a.off_linv) + (int64_t)m * a.n_tiles * kColChunkDev * kRowBlockDev;
+        const int pad = a.n_rb * kRowBlockDev;
+        for (int row = rank + C * warp; row < pad; row += C * nwarps) {
+            const int rb = row / kRowBlockDev, ii = row % kRowBlockDev;
+            const double* Ar = A + (row < n ? local_row_off(row / C, rank) : 0);
+            for (int c = lane; c < (rb + 1) * kRowBlockDev; c += 32)
+                tiles[((size_t)(rb * (rb + 1) + c / kColChunkDev) * kColChunkDev + c % kColChunkDev) * kRowBlockDev + ii] =
+                    row < n && c <= row ? (float)Ar[c] : 0.0f;
+        }
     }
-    // tiles: the owner of a row writes its entries (CTA 0 the padding rows)
-    float* tiles = reinterpret_cast<float*>(a.blob + a.off_linv) + (int64_t)m * a.n_tiles * kColChunkDev * kRowBlockDev;
-    const int64_t total = (int64_t)a.n_tiles * kColChunkDev * kRowBlockDev;
-    for (int64_t e = tid; e < total; e += kClusterThreads) {
-        const int t = (int)(e / (kColChunkDev * kRowBlockDev));
-        const int jj = (int)(e / kRowBlockDev % kColChunkDev), ii = (int)(e % kRowBlockDev);
-        int rb = 0;
-        while ((rb + 1) * (rb + 2) <= t) ++rb;
-        const int cj = t - rb * (rb + 1);
-        const int row = rb * kRowBlockDev + ii, c = cj * kColChunkDev + jj;
-        if (row < n ? row % C != rank : rank != 0) continue;
-        float v = 0.0f;
-        if (row < n && c <= row) v = (float)(W[local_row_off(row / C, rank) + c] * rinv[row]);
-        tiles[e] = v;
-    }
-    cluster.sync();  // CTA 0 has read every CTA's part before any CTA exits
+    cluster.sync();  // no CTA leaves while another may still write to it
 }
 
 constexpr int kMleMaxP = SCOOT_MAX_DIM + 2;  // ln l_1 .. ln l_d, ln s_f^2, ln tau^2
@@ -704,22 +750,6 @@ __global__ void __launch_bounds__(kMleThreads) gp_mle_kernel(const __grid_consta
     if (tid == 0) a.lml[sm] = s_fail ? -INFINITY : lml;
 }
 
-// 1 / v for a normal v > 0 by Newton-Raphson from the hardware's estimate
-// (2^-20, then 2^-40, then beyond 53 bits): four dependent multiply-adds.
-__device__ __forceinline__ double rcp_newton(double v) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
-    y = fma(fma(-v, y, 1.0), y, y);
-    return fma(fma(-v, y, 1.0), y, y);
-}
-
-// Whether v lies in [2^-1000, 2^1000), on the integer pipes: a pivot that
-// can be inverted (a covariance's pivots lie far inside).
-__device__ __forceinline__ bool good_pivot(double v) {
-    const int hi = __double2hiint(v);
-    return hi >= ((1023 - 1000) << 20) && hi < ((1023 + 1000) << 20);
-}
-
 // gp_mle_kernel's fit by a cluster of eight CTAs per (start, objective).
 //
 // One block per fit leaves most SMs idle at the tuning loop's 8 starts, and fp64
@@ -744,7 +774,7 @@ __device__ __forceinline__ bool good_pivot(double v) {
 // n = 128 75.6 against 34.0, 128 fits 75.6 against 67.1.  Larger n than fits (about
 // 300) stay with gp_mle_kernel.  Keeping the squared differences as well cost the
 // second CTA per SM and was slower (25 ms at n = 128).
-constexpr int kMleB = kClusterCTAs;  // pivots per block: one row of a block per CTA
+constexpr int kMleB = kClusterB;
 constexpr int kMleClThreads = 256;
 
 constexpr size_t kMleClTwo = 108 * 1024;  // shared memory of which two CTAs fit an SM
@@ -756,12 +786,7 @@ struct MleClSizes {
 
 inline MleClSizes mle_cl_sizes(int n, int d) {
     MleClSizes z;
-    z.own = 0;
-    for (int r = 0; r < kClusterCTAs; ++r) {
-        const int64_t nl = (n + 1 - r + kClusterCTAs - 1) / kClusterCTAs;  // rows r, r + 8, ... up to n
-        const int64_t e = nl * (r + 1) + (int64_t)kClusterCTAs * nl * (nl - 1) / 2;
-        if (e > z.own) z.own = e;
-    }
+    z.own = cluster_own(n);
     const size_t rows = (size_t)(n + 1 + kClusterCTAs - 1) / kClusterCTAs;
     z.bytes = ((size_t)2 * (n + 1) * kMleB + (size_t)n * d + (size_t)z.own + 2 * (size_t)(n + 1) + rows * kMleB) * sizeof(double);
     z.keep_bytes = 2 * (size_t)z.own * sizeof(double);
@@ -1027,7 +1052,7 @@ extern "C" {
 scoot_status scoot_gp_device_work_bytes(const scoot_gp_layout* L, int64_t* bytes) {
     if (!L || !bytes || !scoot_gp_layout_valid(L)) return SCOOT_EINVAL;
     const int64_t n = L->n, tri = n * (n + 1) / 2;
-    *bytes = 8 * (int64_t)L->n_obj * (n * L->d + tri * (n <= kSmemCholMaxN ? 1 : 2));
+    *bytes = 8 * (int64_t)L->n_obj * (n * L->d + tri * (n <= kOneTriangleN ? 1 : 2));
     return SCOOT_OK;
 }
 
@@ -1109,13 +1134,12 @@ scoot_status scoot_gp_prepare_device(scoot_ctx* ctx, const scoot_param* h_space,
     a.off_scal = L->off_scal;
     a.off_cat = L->off_cat;
     a.off_warp = L->off_warp;
-    const bool in_smem = n <= kSmemCholMaxN;
     const size_t u_bytes = (size_t)M * n * d * sizeof(double);
     const size_t k_bytes = (size_t)M * a.tri * sizeof(double);
     char* ws = static_cast<char*>(work);
     a.U = reinterpret_cast<double*>(ws);
     a.K = reinterpret_cast<double*>(ws + u_bytes);
-    a.W = in_smem ? nullptr : reinterpret_cast<double*>(ws + u_bytes + k_bytes);
+    a.W = n <= kOneTriangleN ? nullptr : reinterpret_cast<double*>(ws + u_bytes + k_bytes);
     a.err = ctx->d_err;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     gp_feat_kernel<<<dim3((n * d + kFeatThreads - 1) / kFeatThreads, M), kFeatThreads, 0, st>>>(a);
@@ -1130,22 +1154,18 @@ scoot_status scoot_gp_prepare_device(scoot_ctx* ctx, const scoot_param* h_space,
     }
     gp_kmat_kernel<<<dim3((unsigned)((a.tri + kKmatThreads - 1) / kKmatThreads), M), kKmatThreads, 0, st>>>(a);
     SCOOT_LAUNCHED(ctx);
-    if (n <= kClusterMaxN) {
-        // rows split over a cluster; shared memory for the CTA with the most entries
-        int64_t own = 0;
-        for (int r = 0; r < kClusterCTAs; ++r) {
-            const int64_t nl = (n - r + kClusterCTAs - 1) / kClusterCTAs;
-            const int64_t e = nl * (r + 1) + (int64_t)kClusterCTAs * nl * (nl - 1) / 2;  // local_row_off(nl, r)
-            if (e > own) own = e;
-        }
-        const size_t csmem = (size_t)8 * n * sizeof(double) + (size_t)2 * own * sizeof(double);
+    int optin = 0;
+    SCOOT_CUDA(ctx, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
+    const size_t csmem = chol_cluster_bytes(n);
+    if (csmem + 4096 <= (size_t)optin) {
         SCOOT_CUDA(ctx, cudaFuncSetAttribute(gp_chol_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)csmem));
-        gp_chol_cluster_kernel<<<M * kClusterCTAs, kClusterThreads, csmem, st>>>(a);
+        gp_chol_cluster_kernel<<<M * kClusterCTAs, kClusterThreads, csmem, st>>>(a, cluster_own(n));
         SCOOT_LAUNCHED(ctx);
         return SCOOT_OK;
     }
-    const size_t smem = (size_t)5 * n * sizeof(double) + (in_smem ? (size_t)2 * a.tri * sizeof(double) : 0);
+    if (!a.W) return scoot_fail(ctx, SCOOT_EUNSUPPORTED, "shared memory of %d bytes is too small", optin);
+    const size_t smem = (size_t)5 * n * sizeof(double);
     SCOOT_CUDA(ctx, cudaFuncSetAttribute(gp_chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     gp_chol_kernel<<<M, kCholThreads, smem, st>>>(a);
     SCOOT_LAUNCHED(ctx);
