@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(kPassThreads, M == 2 ? 4 : 1) fant_pass(const 
             for (int c = 0; c < a.d; ++c) {
                 const float4 f = fm[c];
                 const int kind = (int)f.x;
-                const float ux = feature_of(__ldg(a.cand + (int64_t)f.w * a.ld + i), kind, f.y, f.z);
+                const float ux = feature_of(__ldg(a.cand + (int)f.w * a.ld + i), kind, f.y, f.z);
                 const float up = ups[c];
 #pragma unroll
                 for (int m = 0; m < M; ++m) {

@@ -92,7 +92,7 @@ __device__ __forceinline__ void prefetch_words(uint32_t* wbuf, const uint32_t* c
         for (int q = tid / kTC; q < d; q += kQ) {
             const unsigned dst = (unsigned)__cvta_generic_to_shared(wbuf + q * kTC + s);
             asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst),
-                         "l"(cand + (int64_t)fm[q].w * ld + i) : "memory");
+                         "l"(cand + (int)fm[q].w * ld + i) : "memory");
         }
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
