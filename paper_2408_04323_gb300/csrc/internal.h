@@ -159,7 +159,7 @@ scoot_status scoot_posterior_whitened(scoot_ctx* ctx, const scoot_gp_layout* L, 
 
 // The tensor-core whitened posterior (posterior_tc.cu): the arguments of the
 // SIMT kernel's whitened epilogue plus the split copy of L^{-1}.
-constexpr int kMaxNpadTc = 256;  // output rows held in tensor memory (fp32 columns)
+constexpr int kMaxNpadTc = 256;  // output rows held in tensor memory (fp32 columns) at a time
 struct ScootTcArgs {
     const char* state;
     int64_t off_fmap, off_xs, off_ils, off_alpha, off_scal, off_cat, off_warp, off_linv;
@@ -173,8 +173,14 @@ struct ScootTcArgs {
     int64_t ldo;
     float* vout;      // NULL: moments only
     int32_t by_index; // mean / var at the candidate's index (else at its list position)
+    float* sq;        // n_pad > kMaxNpadTc: [n_obj][n] scratch, by list position
     int32_t accurate; // the covariance's square root and exponential to an fp32 rounding
-    uint8_t* bsplit;  // [M][n_pad / 32][3][n_pad * 64 bytes]
+    uint8_t* bsplit;  // scoot_tc_bsplit_bytes bytes
+    // A group of output rows row0 .. row0 + n_rows - 1 (set by
+    // scoot_posterior_tc): 0 all rows, 1 the first of several groups (its part of
+    // |V|^2 to sq), 2 a middle one (added to it), 3 the last.
+    // Groups past the first accumulate in n_main main accumulators in turn.
+    int32_t row0, n_rows, group, n_main;
     uint32_t* err;
     // Acquisition epilogue (objective 0 only, acq at the candidate's index;
     // mean / var then unused): 0 none, 1 EI (Eq. 6) into acq[i], 2 MACE's
@@ -185,7 +191,7 @@ struct ScootTcArgs {
     float xi, kappa;
 };
 int64_t scoot_tc_bsplit_bytes(int n_pad, int M);
-bool scoot_tc_supported(scoot_ctx* ctx, const ScootTcArgs& a, int DO);
+bool scoot_tc_supported(scoot_ctx* ctx, const ScootTcArgs& a, int DO, bool groups);
 scoot_status scoot_posterior_tc(scoot_ctx* ctx, const ScootTcArgs& a, int DO, cudaStream_t st);
 
 // Monte-Carlo EHVI from moments by list position (ehvi.cu): acq at the

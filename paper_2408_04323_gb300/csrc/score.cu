@@ -674,6 +674,18 @@ ScootTcArgs tc_args(scoot_ctx* ctx, const ScoreArgs& a, int nobj) {
 // Padded ordinal feature count of the kernels (DO).
 int tc_do(const ScoreArgs& a) { return a.n_ord <= 4 ? 4 : a.n_ord <= 8 ? 8 : a.n_ord <= 12 ? 12 : 16; }
 
+// Whether the tensor-core posterior takes the call in groups of rows (more than 256
+// observations): it does beyond two tiles of the fp32 kernel per SM (12 parameters, two
+// objectives, n = 400: 4096 candidates 139 us there against 149, 12288 301 against
+// 150, 2^17 2236 against 801; 5 parameters, one objective, n = 257: 8192 46 against
+// 52, 12288 57 against 52, 2^17 438 against 223).  The covariances take the accurate
+// square root and exponential, so that the error against 64 bits is the fp32 kernel's
+// (0.7 to 1.3 times it over 16 models of 257 to 640 observations, 0.98 on average,
+// mean and variance alike; the largest error of the variance is smaller in 15).
+bool tc_groups(scoot_ctx* ctx, const ScoreArgs& a) {
+    return a.n_rb * kRB > kMaxNpadTc && a.n > (int64_t)sm_count(ctx->device) * 2 * kTC;
+}
+
 // The tensor-core route of the entry points that take moments or an
 // acquisition straight from the posterior, without V: t carries the outputs
 // (mean / var, or the acquisition epilogue) and a.cand / n / ld the pool.
@@ -685,13 +697,17 @@ int tc_do(const ScoreArgs& a) { return a.n_ord <= 4 ? 4 : a.n_ord <= 8 ? 8 : a.n
 scoot_status tc_direct(scoot_ctx* ctx, const ScoreArgs& a, const uint8_t* mask, ScootTcArgs t, int fill_rows,
                        cudaStream_t st, bool* used) {
     *used = false;
-    if (!ctx->tensor_cores || a.n_rb * kRB > kMaxNpadTc) return SCOOT_OK;
+    if (!ctx->tensor_cores) return SCOOT_OK;
     const int DO = tc_do(a);
-    if (!scoot_tc_supported(ctx, t, DO)) return SCOOT_OK;
+    const bool groups = tc_groups(ctx, a);
+    if (groups) t.accurate = 1;
+    if (!scoot_tc_supported(ctx, t, DO, groups)) return SCOOT_OK;
     *used = true;
     const size_t list_bytes = mask ? ((256 + (size_t)a.n * 4 + 255) & ~(size_t)255) : 0;
-    scoot_status s = scoot_workspace(ctx, list_bytes + (size_t)scoot_tc_bsplit_bytes(t.n_pad, t.n_obj));
+    const size_t split_bytes = ((size_t)scoot_tc_bsplit_bytes(t.n_pad, t.n_obj) + 255) & ~(size_t)255;
+    scoot_status s = scoot_workspace(ctx, list_bytes + split_bytes + (groups ? (size_t)t.n_obj * a.n * 4 : 0));
     if (s != SCOOT_OK) return s;
+    if (groups) t.sq = reinterpret_cast<float*>(static_cast<char*>(ctx->ws) + list_bytes + split_bytes);
     if (mask) {
         ScootList lst;
         uint32_t* fill = t.acq_kind ? reinterpret_cast<uint32_t*>(t.acq) : nullptr;
@@ -719,7 +735,7 @@ scoot_status tc_direct(scoot_ctx* ctx, const ScoreArgs& a, const uint8_t* mask, 
 scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* used) {
     *used = false;
     const int M = a.n_obj;
-    if (!ctx->tensor_cores || a.n_rb * kRB > kMaxNpadTc) return SCOOT_OK;
+    if (!ctx->tensor_cores) return SCOOT_OK;
     // One row block (n <= 64) is too little for the tensor cores' pipeline:
     // there the fused kernel stays ahead (n = 64, M = 2, 2^18 candidates 134 us
     // against 160) unless the walk saves more (M = 3, 132 boxes, 2^18: 444 us
@@ -731,12 +747,14 @@ scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* 
     if (a.n_rb == 2 && a.n < 32768) return SCOOT_OK;
     ScootTcArgs t = tc_args(ctx, a, M);
     const int DO = tc_do(a);
-    if (!scoot_tc_supported(ctx, t, DO)) return SCOOT_OK;
+    const bool groups = tc_groups(ctx, a);
+    if (!scoot_tc_supported(ctx, t, DO, groups)) return SCOOT_OK;
     *used = true;
     const size_t list_bytes = a.mask ? ((256 + (size_t)a.n * 4 + 255) & ~(size_t)255) : 0;
     const size_t split_bytes = ((size_t)scoot_tc_bsplit_bytes(t.n_pad, M) + 255) & ~(size_t)255;
     const size_t moment_bytes = ((size_t)M * a.n * 4 + 255) & ~(size_t)255;
-    scoot_status s = scoot_workspace(ctx, list_bytes + split_bytes + 2 * moment_bytes +
+    const size_t sq_bytes = groups ? moment_bytes : 0;
+    scoot_status s = scoot_workspace(ctx, list_bytes + split_bytes + 2 * moment_bytes + sq_bytes +
                                               scoot_ehvi_work_bytes(M, a.n, a.n_boxes, a.n_mc));
     if (s != SCOOT_OK) return s;
     if (a.mask) {
@@ -755,9 +773,10 @@ scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* 
     t.mean = reinterpret_cast<float*>(ws + split_bytes);
     t.var = reinterpret_cast<float*>(ws + split_bytes + moment_bytes);
     t.ldo = a.n;
+    if (groups) t.sq = reinterpret_cast<float*>(ws + split_bytes + 2 * moment_bytes);
     if ((s = scoot_posterior_tc(ctx, t, DO, st)) != SCOOT_OK) return s;
     return scoot_ehvi_listed(ctx, M, t.mean, t.var, a.n, a.n, t.list, t.n_list, a.box_lo, a.box_hi, a.n_boxes, a.eps,
-                             a.n_mc, ws + split_bytes + 2 * moment_bytes, a.acq, st);
+                             a.n_mc, ws + split_bytes + 2 * moment_bytes + sq_bytes, a.acq, st);
 }
 
 }  // namespace
@@ -783,7 +802,7 @@ scoot_status scoot_posterior_whitened(scoot_ctx* ctx, const scoot_gp_layout* L, 
         t.by_index = 0;
         t.bsplit = static_cast<uint8_t*>(tc_work);
         const int DO = tc_do(a);
-        if (scoot_tc_supported(ctx, t, DO)) return scoot_posterior_tc(ctx, t, DO, st);
+        if (scoot_tc_supported(ctx, t, DO, false)) return scoot_posterior_tc(ctx, t, DO, st);
     }
     a.cand = cand;
     a.n = n;
