@@ -736,15 +736,14 @@ scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* 
     *used = false;
     const int M = a.n_obj;
     if (!ctx->tensor_cores) return SCOOT_OK;
-    // One row block (n <= 64) is too little for the tensor cores' pipeline:
-    // there the fused kernel stays ahead (n = 64, M = 2, 2^18 candidates 134 us
-    // against 160) unless the walk saves more (M = 3, 132 boxes, 2^18: 444 us
-    // against 648; 2^15: 113 against 103).
-    // Up to 128 observations it takes 32768 candidates (n = 100, M = 2: 4096
-    // candidates 41 us fused against 43, 16384 48 against 47, 65536 92 against
-    // 71); beyond, the fused kernel loses from 2048 on (n = 200: 78 against 60).
-    if (a.n_rb == 1 && !(a.n >= 65536 && scoot_ehvi_walks(M, a.n, a.n_boxes, a.n_mc))) return SCOOT_OK;
-    if (a.n_rb == 2 && a.n < 32768) return SCOOT_OK;
+    // One row block is little for the tensor cores' pipeline: it takes 65536
+    // candidates and more than 48 observations (8 parameters, M = 2, n = 64: 32768
+    // candidates 34.8 us fused against 34.8, 65536 49.6 against 45.7, 2^18 135 against
+    // 120; n = 40: 2^18 121 against 120; n = 16: 2^18 100 against 112), or the walk to
+    // save more (M = 3, n = 64, 132 boxes: 65536 123 against 115, 2^18 408 against 272).
+    // Beyond, the fused kernel is behind from 1024 candidates on (n = 100, M = 2: 39.0
+    // against 37.4, 65536 90 against 58; n = 128, M = 3: 63 against 61, 173 against 116).
+    if (a.n_rb == 1 && !(a.n >= 65536 && (a.n_obs > 48 || scoot_ehvi_walks(M, a.n, a.n_boxes, a.n_mc)))) return SCOOT_OK;
     ScootTcArgs t = tc_args(ctx, a, M);
     const int DO = tc_do(a);
     const bool groups = tc_groups(ctx, a);
