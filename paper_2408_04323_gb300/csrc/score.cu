@@ -577,18 +577,22 @@ size_t score_smem(const ScoreArgs& a, int epi, int DO) {
     return f * 4;
 }
 
+// Places the staged tables behind score_smem; bytes of shared memory of the kernel.
+size_t place_score(ScoreArgs& a, int epi, int nobj, int DO) {
+    // the categorical table of the objectives this epilogue reads, staged when small
+    const int64_t cat = (int64_t)nobj * a.n_obs * a.n_pat;
+    a.cat_off = (int32_t)(score_smem(a, epi, DO) / 4);
+    a.cat_smem = (a.n_ord < a.d && cat <= kCatSmemMax) ? (int32_t)cat : 0;
+    a.wbuf_off = a.cat_off + ((a.cat_smem + 3) & ~3);
+    return (size_t)(a.wbuf_off + a.d * kTC) * 4;
+}
+
 template <int EPI, int M, int DO>
 scoot_status launch_score_dm(scoot_ctx* ctx, ScoreArgs a, cudaStream_t st) {
-    // the categorical table of the objectives this epilogue reads, staged when small
-    const int nobj = (EPI == kEHVI || EPI == kEHVIX) ? M : ((EPI == kEI || EPI == kMACE) ? 1 : a.n_obj);
-    const int64_t cat = (int64_t)nobj * a.n_obs * a.n_pat;
     auto kern = score_kernel<EPI, M, DO>;
     int optin = 0;
     SCOOT_CUDA(ctx, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
-    a.cat_off = (int32_t)(score_smem(a, EPI, DO) / 4);
-    a.cat_smem = (a.n_ord < a.d && cat <= kCatSmemMax) ? (int32_t)cat : 0;
-    a.wbuf_off = a.cat_off + ((a.cat_smem + 3) & ~3);
-    const size_t smem = (size_t)(a.wbuf_off + a.d * kTC) * 4;
+    const size_t smem = place_score(a, EPI, EPI == kEHVI || EPI == kEHVIX ? M : EPI == kEI || EPI == kMACE ? 1 : a.n_obj, DO);
     if (smem > (size_t)optin)
         return scoot_fail(ctx, SCOOT_EUNSUPPORTED,
                           "score kernel needs %zu bytes of shared memory (n = %d observations, %d boxes), the "
@@ -674,6 +678,14 @@ ScootTcArgs tc_args(scoot_ctx* ctx, const ScoreArgs& a, int nobj) {
 // Padded ordinal feature count of the kernels (DO).
 int tc_do(const ScoreArgs& a) { return a.n_ord <= 4 ? 4 : a.n_ord <= 8 ? 8 : a.n_ord <= 12 ? 12 : 16; }
 
+// Whether the fused kernel has room for the call.  Where it has not, the call is
+// refused there, so no other route takes it.
+bool score_fits(scoot_ctx* ctx, ScoreArgs a, int epi, int nobj) {
+    int optin = 0;
+    return cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device) == cudaSuccess &&
+           place_score(a, epi, nobj, tc_do(a)) <= (size_t)optin;
+}
+
 // Whether the tensor-core posterior takes the call in groups of rows (more than 256
 // observations): it does beyond two tiles of the fp32 kernel per SM (12 parameters, two
 // objectives, n = 400: 4096 candidates 139 us there against 149, 12288 301 against
@@ -701,7 +713,7 @@ scoot_status tc_direct(scoot_ctx* ctx, const ScoreArgs& a, const uint8_t* mask, 
     const int DO = tc_do(a);
     const bool groups = tc_groups(ctx, a);
     if (groups) t.accurate = 1;
-    if (!scoot_tc_supported(ctx, t, DO, groups)) return SCOOT_OK;
+    if (!scoot_tc_supported(ctx, t, DO, groups) || (groups && !score_fits(ctx, a, kWriteMoments, t.n_obj))) return SCOOT_OK;
     *used = true;
     const size_t list_bytes = mask ? ((256 + (size_t)a.n * 4 + 255) & ~(size_t)255) : 0;
     const size_t split_bytes = ((size_t)scoot_tc_bsplit_bytes(t.n_pad, t.n_obj) + 255) & ~(size_t)255;
@@ -744,6 +756,7 @@ scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* 
     // Beyond, the fused kernel is behind from 1024 candidates on (n = 100, M = 2: 39.0
     // against 37.4, 65536 90 against 58; n = 128, M = 3: 63 against 61, 173 against 116).
     if (a.n_rb == 1 && !(a.n >= 65536 && (a.n_obs > 48 || scoot_ehvi_walks(M, a.n, a.n_boxes, a.n_mc)))) return SCOOT_OK;
+    if (!score_fits(ctx, a, kEHVI, M)) return SCOOT_OK;
     ScootTcArgs t = tc_args(ctx, a, M);
     const int DO = tc_do(a);
     const bool groups = tc_groups(ctx, a);

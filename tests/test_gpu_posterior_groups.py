@@ -61,3 +61,18 @@ def test_long_histories(S, ctx, name, n_obs, kernel):  # noqa: F811
         bar = 2 * U32 * (len(lo) + 64) * want[live] + M * 4 * U32 * R * (2 * R) ** (M - 1)
         assert ((got - want)[live].abs() <= bar).all()
     ctx.check()
+
+
+def test_refused_stays_refused(S, ctx):  # noqa: F811
+    """A call whose boxes and samples do not fit beside a long history in the fused
+    kernel is refused with the tensor cores on as with them off."""
+    inst = make_instance("d8-ehvi2", seeds("d8-ehvi2")[0], n_cand=10000)
+    n_obs, M = 640, inst.n_obj
+    L = S.scoot_gp_layout_init(inst.space, n_obs, M, 0)
+    state = torch.zeros(L.bytes, dtype=torch.uint8, device="cuda")
+    cand, acq = dev(inst.cand.view(np.int32)), torch.empty(inst.n_cand, device="cuda")
+    lo, hi, eps = (torch.zeros((k, M), device="cuda") for k in (4000, 4000, 1024))
+    for on in (0, 1):
+        S.scoot_ctx_set_tensor_cores(ctx, on)
+        with pytest.raises(Exception, match="shared memory"):
+            S.scoot_score_ehvi(ctx, L, state, cand, inst.n_cand, lo, hi, eps, acq)
