@@ -44,6 +44,16 @@ scoot_status scoot_workspace(scoot_ctx* ctx, size_t bytes) {
     return SCOOT_OK;
 }
 
+bool scoot_workspace_try(scoot_ctx* ctx, size_t bytes, void* st) {
+    if (bytes <= ctx->ws_bytes) return true;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(static_cast<cudaStream_t>(st), &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone &&
+        scoot_workspace(ctx, bytes) == SCOOT_OK)
+        return true;
+    cudaGetLastError();  // the caller goes on without it
+    return false;
+}
+
 static scoot_status record_event(scoot_ctx* ctx, void* st) {
     const size_t k = ctx->mark_kind.size();
     if (k >= (size_t)SCOOT_MAX_MARKS + 1) return SCOOT_OK;  // later launches are not timed

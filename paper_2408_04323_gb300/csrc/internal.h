@@ -47,6 +47,9 @@ void scoot_host_parallel(int count, const std::function<void(int)>& fn);
 scoot_status scoot_enter(scoot_ctx* ctx);
 // Ensure at least `bytes` of workspace (synchronising the device if it grows).
 scoot_status scoot_workspace(scoot_ctx* ctx, size_t bytes);
+// Whether a call on stream st can have `bytes` of workspace; grows it if needed, but
+// not while st is being captured.  For routes with another that needs less.
+bool scoot_workspace_try(scoot_ctx* ctx, size_t bytes, void* st);
 
 static inline bool scoot_aligned16(const void* p) {
     return (reinterpret_cast<uintptr_t>(p) & 15u) == 0;

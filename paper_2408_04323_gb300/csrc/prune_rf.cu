@@ -565,14 +565,11 @@ scoot_status scoot_rf_predict(scoot_ctx* ctx, const scoot_forest_layout* L, cons
     // against 52, 63 against 64, 161 against 155; 2^18 97 against 88, 112 against 107, 299 against 263;
     // 2^20 380 against 289, 439 against 353, 1180 against 894; 2^22 4967 against 3479.
     // With a mask about half of the pool is walked.
-    const bool ranked = L->n_nodes <= kRankNodes && L->leaf_scale <= kRankVotes &&
-                        n * L->n_trees * (L->max_depth + 1) >= (mask ? kRankFrom * 2 : kRankFrom);
     const size_t list_bytes = mask ? ((256 + (size_t)n * 4 + 255) & ~(size_t)255) : 0;
     const size_t node_bytes = ((size_t)L->n_nodes * 8 + 255) & ~(size_t)255;
-    if (ranked) {
-        s = scoot_workspace(ctx, list_bytes + node_bytes + (size_t)L->d * kRankThr * 4 + 256);
-        if (s != SCOOT_OK) return s;
-    }
+    const bool ranked = L->n_nodes <= kRankNodes && L->leaf_scale <= kRankVotes &&
+                        n * L->n_trees * (L->max_depth + 1) >= (mask ? kRankFrom * 2 : kRankFrom) &&
+                        scoot_workspace_try(ctx, list_bytes + node_bytes + (size_t)L->d * kRankThr * 4 + 256, st);
     if (mask) {
         // Walk only the candidates still in play; the others get 0 votes.
         ScootList lst;

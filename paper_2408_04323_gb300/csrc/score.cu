@@ -714,10 +714,12 @@ scoot_status tc_direct(scoot_ctx* ctx, const ScoreArgs& a, const uint8_t* mask, 
     const bool groups = tc_groups(ctx, a);
     if (groups) t.accurate = 1;
     if (!scoot_tc_supported(ctx, t, DO, groups) || (groups && !score_fits(ctx, a, kWriteMoments, t.n_obj))) return SCOOT_OK;
-    *used = true;
     const size_t list_bytes = mask ? ((256 + (size_t)a.n * 4 + 255) & ~(size_t)255) : 0;
     const size_t split_bytes = ((size_t)scoot_tc_bsplit_bytes(t.n_pad, t.n_obj) + 255) & ~(size_t)255;
-    scoot_status s = scoot_workspace(ctx, list_bytes + split_bytes + (groups ? (size_t)t.n_obj * a.n * 4 : 0));
+    const size_t bytes = list_bytes + split_bytes + (groups ? (size_t)t.n_obj * a.n * 4 : 0);
+    if (groups && !scoot_workspace_try(ctx, bytes, st)) return SCOOT_OK;
+    *used = true;
+    scoot_status s = scoot_workspace(ctx, bytes);
     if (s != SCOOT_OK) return s;
     if (groups) t.sq = reinterpret_cast<float*>(static_cast<char*>(ctx->ws) + list_bytes + split_bytes);
     if (mask) {
@@ -736,14 +738,53 @@ scoot_status tc_direct(scoot_ctx* ctx, const ScoreArgs& a, const uint8_t* mask, 
     return scoot_posterior_tc(ctx, t, DO, st);
 }
 
-// The route of scoot_score_ehvi through the tensor cores: the posterior's
-// moments by list position into the workspace, then the EHVI of ehvi.cu.
-// Workspace: the compacted list (when masked), the split copy of L^{-1}, the
-// moments and the EHVI's scratch, reserved whole before the list is written.
+// The moments of a call's live candidates on the tensor cores, by list position or
+// by index, into the workspace: the compacted list (when masked, -inf for the
+// others' acquisition), the split copy of L^{-1}, the moments, the groups' sums and
+// `extra` bytes for the caller (*work), reserved whole before the list is written
+// (where they cannot be had the fused kernel, which needs less, takes the call).
 // *used as for tc_direct.  The covariances take the accurate square root and
 // exponential (7% of the posterior's time): the acquisition's error against 64
-// bits is then that of the fused kernel (0.7 to 1.2 times it over 21 models of 70
-// to 256 observations, 1.0 on average; 1.1 without).
+// bits is then that of the fused kernel (over 64 models of 70 to 256 observations,
+// Monte-Carlo and closed form, 0.98 times it on average and 0.5 to 1.7 in one
+// model; 1.1 without).
+scoot_status tc_moments(scoot_ctx* ctx, const ScoreArgs& a, ScootTcArgs& t, int by_index, size_t extra, cudaStream_t st,
+                        char** work, bool* used) {
+    *used = false;
+    const int M = a.n_obj, DO = tc_do(a);
+    const bool groups = tc_groups(ctx, a);
+    if (!scoot_tc_supported(ctx, t, DO, groups)) return SCOOT_OK;
+    const size_t list_bytes = a.mask ? ((256 + (size_t)a.n * 4 + 255) & ~(size_t)255) : 0;
+    const size_t split_bytes = ((size_t)scoot_tc_bsplit_bytes(t.n_pad, M) + 255) & ~(size_t)255;
+    const size_t moment_bytes = ((size_t)M * a.n * 4 + 255) & ~(size_t)255;
+    const size_t sq_bytes = groups ? moment_bytes : 0;
+    if (!scoot_workspace_try(ctx, list_bytes + split_bytes + 2 * moment_bytes + sq_bytes + extra, st)) return SCOOT_OK;
+    *used = true;
+    scoot_status s;
+    if (a.mask) {
+        ScootList lst;
+        if ((s = scoot_compact(ctx, a.mask, a.n, reinterpret_cast<uint32_t*>(a.acq), 0xFF800000u, st, &lst)) != SCOOT_OK)
+            return s;
+        t.list = lst.list;
+        t.n_list = lst.count;
+    }
+    char* ws = static_cast<char*>(ctx->ws) + list_bytes;
+    t.cand = a.cand;
+    t.n = a.n;
+    t.ld = a.ld;
+    t.accurate = 1;
+    t.by_index = by_index;
+    t.bsplit = reinterpret_cast<uint8_t*>(ws);
+    t.mean = reinterpret_cast<float*>(ws + split_bytes);
+    t.var = reinterpret_cast<float*>(ws + split_bytes + moment_bytes);
+    t.ldo = a.n;
+    if (groups) t.sq = reinterpret_cast<float*>(ws + split_bytes + 2 * moment_bytes);
+    *work = ws + split_bytes + 2 * moment_bytes + sq_bytes;
+    return scoot_posterior_tc(ctx, t, DO, st);
+}
+
+// The route of scoot_score_ehvi through the tensor cores: the posterior's moments by
+// list position, then the EHVI of ehvi.cu.
 scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* used) {
     *used = false;
     const int M = a.n_obj;
@@ -758,37 +799,61 @@ scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* 
     if (a.n_rb == 1 && !(a.n >= 65536 && (a.n_obs > 48 || scoot_ehvi_walks(M, a.n, a.n_boxes, a.n_mc)))) return SCOOT_OK;
     if (!score_fits(ctx, a, kEHVI, M)) return SCOOT_OK;
     ScootTcArgs t = tc_args(ctx, a, M);
-    const int DO = tc_do(a);
-    const bool groups = tc_groups(ctx, a);
-    if (!scoot_tc_supported(ctx, t, DO, groups)) return SCOOT_OK;
-    *used = true;
-    const size_t list_bytes = a.mask ? ((256 + (size_t)a.n * 4 + 255) & ~(size_t)255) : 0;
-    const size_t split_bytes = ((size_t)scoot_tc_bsplit_bytes(t.n_pad, M) + 255) & ~(size_t)255;
-    const size_t moment_bytes = ((size_t)M * a.n * 4 + 255) & ~(size_t)255;
-    const size_t sq_bytes = groups ? moment_bytes : 0;
-    scoot_status s = scoot_workspace(ctx, list_bytes + split_bytes + 2 * moment_bytes + sq_bytes +
-                                              scoot_ehvi_work_bytes(M, a.n, a.n_boxes, a.n_mc));
-    if (s != SCOOT_OK) return s;
-    if (a.mask) {
-        ScootList lst;
-        if ((s = scoot_compact(ctx, a.mask, a.n, reinterpret_cast<uint32_t*>(a.acq), 0xFF800000u, st, &lst)) != SCOOT_OK)
-            return s;
-        t.list = lst.list;
-        t.n_list = lst.count;
-    }
-    char* ws = static_cast<char*>(ctx->ws) + list_bytes;
-    t.cand = a.cand;
-    t.n = a.n;
-    t.ld = a.ld;
-    t.accurate = 1;
-    t.bsplit = reinterpret_cast<uint8_t*>(ws);
-    t.mean = reinterpret_cast<float*>(ws + split_bytes);
-    t.var = reinterpret_cast<float*>(ws + split_bytes + moment_bytes);
-    t.ldo = a.n;
-    if (groups) t.sq = reinterpret_cast<float*>(ws + split_bytes + 2 * moment_bytes);
-    if ((s = scoot_posterior_tc(ctx, t, DO, st)) != SCOOT_OK) return s;
+    char* work;
+    const scoot_status s = tc_moments(ctx, a, t, 0, scoot_ehvi_work_bytes(M, a.n, a.n_boxes, a.n_mc), st, &work, used);
+    if (!*used || s != SCOOT_OK) return s;
     return scoot_ehvi_listed(ctx, M, t.mean, t.var, a.n, a.n, t.list, t.n_list, a.box_lo, a.box_hi, a.n_boxes, a.eps,
-                             a.n_mc, ws + split_bytes + 2 * moment_bytes + sq_bytes, a.acq, st);
+                             a.n_mc, work, a.acq, st);
+}
+
+size_t exact_smem(const ScoreArgs& a, int n_obj) {
+    return ((size_t)a.psi_rows * kAcqThreads + ((a.psi_rows + 3) & ~3) + (size_t)a.n_boxes * n_obj) * 4;
+}
+
+// The closed-form EHVI of the moments a.mean and a.var (by index).
+scoot_status launch_exact(scoot_ctx* ctx, const ScoreArgs& a, int n_obj, cudaStream_t st) {
+    const size_t smem = exact_smem(a, n_obj);
+    int64_t blocks = (a.n + kAcqThreads - 1) / kAcqThreads;
+    auto go = [&](auto kern) -> scoot_status {
+        SCOOT_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        int per_sm = 0;
+        SCOOT_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kAcqThreads, smem));
+        if (per_sm < 1) return scoot_fail(ctx, SCOOT_EUNSUPPORTED, "exact EHVI kernel does not fit");
+        const int64_t cap = (int64_t)sm_count(ctx->device) * per_sm;
+        if (blocks > cap) blocks = cap;
+        kern<<<(unsigned)blocks, kAcqThreads, smem, st>>>(a);
+        SCOOT_LAUNCHED(ctx);
+        return SCOOT_OK;
+    };
+    switch (n_obj) {
+    case 2: return go(ehvix_kernel<2>);
+    case 3: return go(ehvix_kernel<3>);
+    default: return go(ehvix_kernel<4>);
+    }
+}
+
+// The route of scoot_score_ehvi_exact through the tensor cores.
+scoot_status tc_exact(scoot_ctx* ctx, ScoreArgs a, cudaStream_t st, bool* used) {
+    *used = false;
+    // Whole rounds, M = 2: 8 parameters, warped, n = 75: 32768 candidates 78 us fused
+    // against 83, 65536 98 against 93, 2^18 216 against 174; n = 64: no gain up to 2^18
+    // (141 against 140); n = 256: 16384 121 against 90, 2^18 655 against 251.
+    if (!ctx->tensor_cores || a.n_rb == 1 || a.n < (a.n_rb == 2 ? 65536 : 16384)) return SCOOT_OK;
+    if (!score_fits(ctx, a, kEHVIX, a.n_obj)) return SCOOT_OK;
+    int optin = 0;
+    SCOOT_CUDA(ctx, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
+    if (exact_smem(a, a.n_obj) + 1024 > (size_t)optin) return SCOOT_OK;
+    ScootTcArgs t = tc_args(ctx, a, a.n_obj);
+    char* work;
+    const scoot_status s = tc_moments(ctx, a, t, 1, 0, st, &work, used);
+    if (!*used || s != SCOOT_OK) return s;
+    a.mean = t.mean;
+    a.var = t.var;
+    a.ldo = a.n;
+    a.list = t.list;
+    a.n_list = t.n_list;
+    a.err = ctx->d_err;
+    return launch_exact(ctx, a, a.n_obj, st);
 }
 
 }  // namespace
@@ -959,7 +1024,6 @@ scoot_status scoot_acq_ehvi_exact(scoot_ctx* ctx, const float* mean, const float
     a.n = n;
     a.acq = acq;
     a.err = ctx->d_err;
-    const size_t smem = ((size_t)a.psi_rows * kAcqThreads + ((a.psi_rows + 3) & ~3) + (size_t)n_boxes * n_obj) * 4;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (mask) {
         ScootList lst;
@@ -968,23 +1032,7 @@ scoot_status scoot_acq_ehvi_exact(scoot_ctx* ctx, const float* mean, const float
         a.list = lst.list;
         a.n_list = lst.count;
     }
-    int64_t blocks = (n + kAcqThreads - 1) / kAcqThreads;
-    auto go = [&](auto kern) -> scoot_status {
-        SCOOT_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        int per_sm = 0;
-        SCOOT_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kAcqThreads, smem));
-        if (per_sm < 1) return scoot_fail(ctx, SCOOT_EUNSUPPORTED, "exact EHVI kernel does not fit");
-        const int64_t cap = (int64_t)sm_count(ctx->device) * per_sm;
-        if (blocks > cap) blocks = cap;
-        kern<<<(unsigned)blocks, kAcqThreads, smem, st>>>(a);
-        SCOOT_LAUNCHED(ctx);
-        return SCOOT_OK;
-    };
-    switch (n_obj) {
-    case 2: return go(ehvix_kernel<2>);
-    case 3: return go(ehvix_kernel<3>);
-    default: return go(ehvix_kernel<4>);
-    }
+    return launch_exact(ctx, a, n_obj, st);
 }
 
 scoot_status scoot_score_ehvi_exact(scoot_ctx* ctx, const scoot_gp_layout* L, const void* state,
@@ -1004,7 +1052,11 @@ scoot_status scoot_score_ehvi_exact(scoot_ctx* ctx, const scoot_gp_layout* L, co
     a.ld = ld;
     a.mask = mask;
     a.acq = acq;
-    return dispatch_m<kEHVIX>(ctx, a, L->n_obj, static_cast<cudaStream_t>(stream));
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    bool used = false;
+    s = tc_exact(ctx, a, st, &used);
+    if (used || s != SCOOT_OK) return s;
+    return dispatch_m<kEHVIX>(ctx, a, L->n_obj, st);
 }
 
 scoot_status scoot_score_ei(scoot_ctx* ctx, const scoot_gp_layout* L, const void* state,

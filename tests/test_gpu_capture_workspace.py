@@ -1,0 +1,51 @@
+"""Calls without a mask need no workspace on their fused kernels: captured as a
+context's first call, when nothing may be allocated, they still run, and replay."""
+import numpy as np
+import pytest
+
+from workloads import Stream, make_instance, seeds
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("call", ["ehvi", "exact"])
+def test_first_call_captured(call):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2408_04323_gb300 as pkg
+    pkg.build()
+    from paper_2408_04323_gb300 import scoot as S
+    inst = make_instance("d10-ehvi3", seeds("d10-ehvi3")[0], n_cand=16384)
+    n, M = inst.n_cand, inst.n_obj
+    L = S.scoot_gp_layout_init(inst.space, inst.n_obs, M, 0)
+    blob, _ = S.scoot_gp_prepare(inst.space, inst.x_obs, inst.y_obs, inst.lengthscale, inst.signal_var, inst.noise_var, L)
+    lo, hi, _ = S.scoot_boxes_build(inst.y_obs, inst.ref)
+    grid, n_grid, corner = S.scoot_boxes_index(lo, hi)
+
+    def dev(a):
+        return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    state, cand, lo, hi, grid = dev(blob), dev(inst.cand.view(np.int32)), dev(lo), dev(hi), dev(grid)
+    corner, eps = dev(corner.view(np.int32)), dev(Stream(1, "eps").normal(32 * M).reshape(32, M).astype(np.float32))
+
+    def run(ctx, acq):
+        if call == "ehvi":
+            S.scoot_score_ehvi(ctx, L, state, cand, n, lo, hi, eps, acq)
+        else:
+            S.scoot_score_ehvi_exact(ctx, L, state, cand, n, grid, n_grid, corner, acq)
+    want, got = torch.empty(n, device="cuda"), torch.full((n,), 7.0, device="cuda")
+    with S.Context(0) as fused:  # (also loads the kernels)
+        S.scoot_ctx_set_tensor_cores(fused, 0)
+        run(fused, want)
+        fused.check()
+    with S.Context(0) as ctx:
+        graph = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph):
+            run(ctx, got)
+        for _ in range(2):
+            got.fill_(7.0)
+            graph.replay()
+            torch.cuda.synchronize()
+            ctx.check()
+            assert torch.equal(got, want)  # the fused kernel took the call
