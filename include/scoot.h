@@ -12,7 +12,7 @@
  *   scoot_acq_ei         expected improvement, Eq. (6)
  *   scoot_acq_ehvi       Monte-Carlo expected hypervolume improvement, Eq. (7)
  *   scoot_score_ei       posterior + EI in one pass
- *   scoot_score_ehvi     posterior + EHVI in one kernel
+ *   scoot_score_ehvi     posterior + EHVI in one call
  *   scoot_score_ehvi_exact  posterior + exact EHVI (independent Gaussians)
  *   scoot_select_topq    top-q for parallel suggestion (Section 4.7)
  *   scoot_score_mace     posterior + UCB, PI, EI for MACE (Section 4.5)
@@ -155,12 +155,15 @@ scoot_status scoot_ctx_workspace_bytes(const scoot_ctx* ctx, int64_t* bytes);
 scoot_status scoot_ctx_set_timing(scoot_ctx* ctx, int32_t enable);
 
 /* Tensor cores for the posterior (on by default).  With enable != 0 the
- * posterior of scoot_gp_posterior, scoot_score_ei, scoot_score_mace and
- * scoot_suggest_fantasy / scoot_fantasy_begin computes
- * V = L^{-1} k(X, x) on the tcgen05 tensor cores when the padded observation
- * count is at most 256 and the state fits a block's shared memory: each fp32
- * operand split into three bf16 parts, six part products accumulated in fp32
- * (the m l, l m, l l products, of order 2^-24, dropped); with enable == 0,
+ * posterior of scoot_gp_posterior, scoot_score_ei, scoot_score_mace,
+ * scoot_score_ehvi, scoot_score_ehvi_exact and scoot_suggest_fantasy /
+ * scoot_fantasy_begin computes V = L^{-1} k(X, x) on the tcgen05 tensor cores
+ * when the state fits a block's shared memory: each fp32 operand split into
+ * three bf16 parts, six part products accumulated in fp32 (the m l, l m, l l
+ * products, of order 2^-24, dropped).  Padded observation counts above 256 are
+ * taken in groups of rows where V is not kept (not in the fantasy calls) and the
+ * pool is large; scoot_score_ehvi and scoot_score_ehvi_exact take the tensor
+ * cores where they are faster than their fused fp32 kernels.  With enable == 0,
  * or outside those limits, the fp32 SIMT product.  The paper has no
  * counterpart (Section 4.3 states the posterior, not how it is computed). */
 scoot_status scoot_ctx_set_tensor_cores(scoot_ctx* ctx, int32_t enable);
@@ -402,16 +405,18 @@ scoot_status scoot_acq_ehvi(scoot_ctx* ctx, const float* mean, const float* var,
 
 /* scoot_gp_posterior followed by scoot_acq_ei, in one pass, without
  * writing mean or variance (objective 0; y_best is the state's best
- * observed value of objective 0).  With the context's tensor cores on and
- * at most 256 observations the pass is the tensor-core posterior with an EI
- * epilogue (after a small kernel that splits L^{-1} into bf16 parts in the
- * context workspace), else one fused fp32 kernel; where mask[i] == 0,
+ * observed value of objective 0).  With the context's tensor cores on the
+ * pass is the tensor-core posterior with an EI epilogue (after a small kernel
+ * that splits L^{-1} into bf16 parts in the context workspace; above 256
+ * observations a pass per group of rows), else one fused fp32 kernel; where mask[i] == 0,
  * acq[i] = -inf. */
 scoot_status scoot_score_ei(scoot_ctx* ctx, const scoot_gp_layout* layout, const void* state,
                             const uint32_t* cand, int64_t n, int64_t ld, const uint8_t* mask,
                             float xi, float* acq, void* stream);
 
-/* scoot_gp_posterior followed by scoot_acq_ehvi, in one kernel. */
+/* scoot_gp_posterior followed by scoot_acq_ehvi, in one call: one fused kernel,
+ * or on the tensor cores (from 65 observations, or large pools) the moments into
+ * the context workspace and a kernel that visits the boxes. */
 scoot_status scoot_score_ehvi(scoot_ctx* ctx, const scoot_gp_layout* layout, const void* state,
                               const uint32_t* cand, int64_t n, int64_t ld, const uint8_t* mask,
                               const float* box_lo, const float* box_hi, int32_t n_boxes,
@@ -435,7 +440,9 @@ scoot_status scoot_acq_ehvi_exact(scoot_ctx* ctx, const float* mean, const float
                                   int32_t grid_cap, const int32_t* h_n_grid, const uint32_t* corner,
                                   int32_t n_boxes, float* acq, void* stream);
 
-/* scoot_gp_posterior followed by scoot_acq_ehvi_exact, in one kernel. */
+/* scoot_gp_posterior followed by scoot_acq_ehvi_exact, in one call: one fused
+ * kernel, or in larger pools the moments from the tensor cores and the closed
+ * form over them. */
 scoot_status scoot_score_ehvi_exact(scoot_ctx* ctx, const scoot_gp_layout* layout, const void* state,
                                     const uint32_t* cand, int64_t n, int64_t ld, const uint8_t* mask,
                                     const float* grid, int32_t grid_cap, const int32_t* h_n_grid,

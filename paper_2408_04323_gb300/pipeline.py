@@ -233,7 +233,9 @@ class ScoringRound:
         """Library kernel launches of one run(): prune, compaction, forest walk, then
         either compaction + fused score + two top-q passes, or (fantasies)
         compaction + posterior + the front's boxes + per pick a pass (downdate,
-        EHVI, block argmax) and the pick's terms."""
+        EHVI, block argmax) and the pick's terms.  At least: the tensor-core
+        posterior adds the split of L^{-1}, a large pool's forest the ranking of
+        its thresholds, EHVI on the tensor cores the boxes' walk."""
         if self.inp.acq == "mace":
             return 10  # prune, compaction, forest, compaction, score, five Pareto kernels
         if not self.inp.fantasy:
