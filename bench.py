@@ -53,11 +53,10 @@ KERNEL_FILES = {"prune": ["prune_rf.cu"], "rf": ["prune_rf.cu"],
 TRAFFIC = {
     # d12-fantasy: captured on a 2^20 pool of the same workload, scaled to the 2^22 launch by its
     # live candidates (x 4.0025; fant_pass and the posterior) or its pool size (x 4; prune, forest)
-    ("fant_pass", "d12-fantasy"): {"bytes": 3561900000, "sha": "3e1f5ef592e904d1"},
-    ("posterior", "d12-fantasy"): {"bytes": 3442600000, "sha": "fef1b84575f65e56"},
-    ("rf", "d12-fantasy"): {"bytes": 227260000, "sha": "df8284c4f1f3b084"},
-    ("prune", "d12-fantasy"): {"bytes": 100700000, "sha": "df8284c4f1f3b084"},
-    ("score", "d10-ehvi3"): {"bytes": 44739000, "sha": "6b2aeb7ebc645ff4"},
+    ("fant_pass", "d12-fantasy"): {"bytes": 3562000000, "sha": "debd6c98ff2ef39c"},
+    ("posterior", "d12-fantasy"): {"bytes": 3441200000, "sha": "36bb65e51b734d88"},
+    ("rf", "d12-fantasy"): {"bytes": 210590000, "sha": "9160ae57ca73ba4f"},
+    ("prune", "d12-fantasy"): {"bytes": 100700000, "sha": "9160ae57ca73ba4f"},
 }
 
 
