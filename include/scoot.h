@@ -441,8 +441,8 @@ scoot_status scoot_acq_ehvi_exact(scoot_ctx* ctx, const float* mean, const float
                                   int32_t n_boxes, float* acq, void* stream);
 
 /* scoot_gp_posterior followed by scoot_acq_ehvi_exact, in one call: one fused
- * kernel, or in larger pools the moments from the tensor cores and the closed
- * form over them. */
+ * kernel, or from 129 observations on in larger pools the moments from the
+ * tensor cores and the closed form over them. */
 scoot_status scoot_score_ehvi_exact(scoot_ctx* ctx, const scoot_gp_layout* layout, const void* state,
                                     const uint32_t* cand, int64_t n, int64_t ld, const uint8_t* mask,
                                     const float* grid, int32_t grid_cap, const int32_t* h_n_grid,

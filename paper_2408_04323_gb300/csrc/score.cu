@@ -835,10 +835,12 @@ scoot_status launch_exact(scoot_ctx* ctx, const ScoreArgs& a, int n_obj, cudaStr
 // The route of scoot_score_ehvi_exact through the tensor cores.
 scoot_status tc_exact(scoot_ctx* ctx, ScoreArgs a, cudaStream_t st, bool* used) {
     *used = false;
-    // Whole rounds, M = 2: 8 parameters, warped, n = 75: 32768 candidates 78 us fused
-    // against 83, 65536 98 against 93, 2^18 216 against 174; n = 64: no gain up to 2^18
-    // (141 against 140); n = 256: 16384 121 against 90, 2^18 655 against 251.
-    if (!ctx->tensor_cores || a.n_rb == 1 || a.n < (a.n_rb == 2 ? 65536 : 16384)) return SCOOT_OK;
+    // Whole rounds, M = 2: 5 parameters, n = 200: 16384 candidates 114 us fused against
+    // 85, 2^18 883 against 358; 8 parameters, n = 256: 121 against 90, 655 against 251.
+    // Up to 128 observations there is less to gain (n = 75: 65536 98 against 93, 2^18 216
+    // against 174), and at n = 70 the error against 64 bits was 1.04 times the fused
+    // kernel's over 8 models (up to 1.7 in one; n = 180 and 256: 0.97).
+    if (!ctx->tensor_cores || a.n_rb <= 2 || a.n < 16384) return SCOOT_OK;
     if (!score_fits(ctx, a, kEHVIX, a.n_obj)) return SCOOT_OK;
     int optin = 0;
     SCOOT_CUDA(ctx, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
