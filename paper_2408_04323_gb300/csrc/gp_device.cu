@@ -412,7 +412,7 @@ gp_chol_cluster_kernel(const __grid_constant__ GpPrepArgs a, int64_t own) {
             }
         }
     };
-    __syncthreads();
+    cluster.sync();  // every CTA has started: its shared memory may be written
     push(0);
     cluster.sync();
     for (int kb = 0; kb < n; kb += B) {
@@ -863,6 +863,7 @@ gp_mle_cluster_kernel(const __grid_constant__ MleArgs a, int64_t own, int keep) 
             }
         }
     };
+    cluster.sync();  // every CTA has started: its shared memory may be written
     double lml = 0.0;
     for (int it = 0; it <= a.steps; ++it) {
         __syncthreads();
