@@ -346,6 +346,101 @@ __device__ __forceinline__ bool good_pivot(double v) {
     return hi >= ((1023 - 1000) << 20) && hi < ((1023 + 1000) << 20);
 }
 
+// What the eliminations of a block's pivots need of the pivot rows.
+struct PanelPivots {
+    double col[kClusterB][kClusterB];  // [p][c > p] entry (kb + c, kb + p) when pivot p is reached
+    double rcp[kClusterB], piv[kClusterB];
+};
+
+// Eliminates pivots kb .. kb + be - 1 from the panel P ([n + 1][8], row j the
+// entries of row or column j of the matrix in the block's columns) one after the
+// other, by a block of kClusterThreads:
+//   t = P_jp / A_pp,  P_jc -= t A_cp  for c > p,
+// the operations of an unblocked elimination in its order, so no block is inverted
+// (multiplying by the inverse of a block of repeated observations cost 1e3 to 1e7
+// times the error).  The rows of the block are replaced by those that its columns of
+// the identity end as.  gs[li][p] = t for the CTA's own rows j = rank + 8 li, the
+// block's own row among them; rows before kb only if all_rows.  On return (after the
+// caller's next __syncthreads) A_ij of two other rows loses gs[i] . P[j].
+// Warp 0 runs the chain of pivots on the block's 8 rows and the identity's, in
+// registers; the other warps follow it on their rows pivot by pivot (named barriers 1
+// to 8), so that the panel costs little beyond that chain.
+__device__ __forceinline__ void eliminate_panel(double* P, double* gs, PanelPivots& s, int* fail, int n, int kb, int be,
+                                                int rank, bool all_rows) {
+    constexpr int C = kClusterCTAs, B = kClusterB, kFirst = kClusterThreads - 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rows = n + 1 - be;  // rows outside the block
+    double y[B], t[B];
+#pragma unroll
+    for (int p = 0; p < B; ++p) t[p] = 0.0;
+    auto step = [&](int p, double rcp, const double* col) {
+        t[p] = y[p] * rcp;
+#pragma unroll
+        for (int c = 0; c < B; ++c)
+            if (c > p) y[c] = fma(-t[p], col[c], y[c]);
+    };
+    auto load = [&](int j) {
+#pragma unroll
+        for (int c = 0; c < B; ++c) y[c] = P[(size_t)j * B + c];
+    };
+    auto store = [&](int j) {
+#pragma unroll
+        for (int c = 0; c < B; ++c) P[(size_t)j * B + c] = y[c];
+        if (j % C == rank && (all_rows || j >= kb)) {
+#pragma unroll
+            for (int c = 0; c < B; ++c) gs[(j / C) * B + c] = t[c];
+        }
+    };
+    auto row_of = [&](int k) { return k < kb ? k : k + be; };
+    if (warp == 0) {  // lanes 0 .. 7: the block's rows; 8 .. 15: the identity's
+        const int r = lane % B;
+#pragma unroll
+        for (int c = 0; c < B; ++c) y[c] = lane < B ? (r < be ? P[(size_t)(kb + r) * B + c] : 0.0) : (r == c ? 1.0 : 0.0);
+#pragma unroll
+        for (int p = 0; p < B; ++p) {
+            if (p >= be) break;
+            const double v = __shfl_sync(0xffffffffu, y[p], p);
+            double col[B];
+#pragma unroll
+            for (int c = 0; c < B; ++c) col[c] = c > p ? __shfl_sync(0xffffffffu, y[c], p) : 0.0;
+            const bool ok = good_pivot(v);
+            const double rcp = ok ? rcp_newton(v) : 0.0;
+            if (lane == 0) {
+                if (!ok) *fail = 1;
+                s.piv[p] = v;
+                s.rcp[p] = rcp;
+#pragma unroll
+                for (int c = 0; c < B; ++c)
+                    if (c > p) s.col[p][c] = col[c];
+            }
+            __syncwarp();
+            asm volatile("bar.arrive %0, %1;" ::"r"(p + 1), "n"(kClusterThreads) : "memory");
+            step(p, rcp, col);
+        }
+        if (lane >= B && lane < B + be) store(kb + r);
+    } else {  // (warp 4 shares warp 0's scheduler, so it comes last)
+        const int k = (warp < 4 ? warp - 1 : warp == 4 ? 6 : warp - 2) * 32 + lane, j = row_of(k);
+        if (k < rows) load(j);
+#pragma unroll
+        for (int p = 0; p < B; ++p) {
+            if (p >= be) break;
+            asm volatile("bar.sync %0, %1;" ::"r"(p + 1), "n"(kClusterThreads) : "memory");
+            if (k < rows) step(p, s.rcp[p], s.col[p]);
+        }
+        if (k < rows) store(j);
+    }
+    for (int k = kFirst + tid; k < rows; k += kClusterThreads) {  // the rows that are left
+        const int j = row_of(k);
+        load(j);
+#pragma unroll
+        for (int p = 0; p < B; ++p) {
+            if (p >= be) break;
+            step(p, s.rcp[p], s.col[p]);
+        }
+        store(j);
+    }
+}
+
 // Bytes of shared memory of gp_chol_cluster_kernel.
 inline size_t chol_cluster_bytes(int n) {
     const size_t rows = (size_t)(n + 1 + kClusterCTAs - 1) / kClusterCTAs;
@@ -356,16 +451,17 @@ inline size_t chol_cluster_bytes(int n) {
 // eight pivots.  CTA r owns rows i = r (mod 8) of K + tau^2 I, augmented by row n,
 // which holds y^T.  The elimination is in place: entry t of row i holds A_it
 // before pivot t and W_it, the elimination of the identity, after it.  A block of
-// pivots kb .. kb + 7 with D = A_kb..kb+7 = L_D L_D^T (X = L_D^{-1}) finishes its
-// rows of L^{-1}, X W, and takes from every later row i
-//   A_ij -= g_i . A_j,block,   W_it -= g_i . W_block,t,   g_i = A_i,block D^{-1}
-// so that row n ends as -alpha^T = -y^T (K + tau^2 I)^{-1}.  What a block needs of
-// other CTAs' rows is one panel of eight values per row or column, which every
-// CTA pushes its part of into all eight CTAs' shared memory: one cluster barrier
-// per eight pivots (one per pivot and two triangles before).  Each CTA
-// factorises the 8 x 8 block for itself.
+// pivots kb .. kb + 7 finishes its rows of L^{-1} and takes from every later row i
+//   A_ij -= g_i . P_j,   W_it -= g_i . P_t
+// with the panel P and the multipliers g of eliminate_panel, so that row n ends as
+// -alpha^T = -y^T (K + tau^2 I)^{-1}.  What a block needs of other CTAs' rows is
+// that panel, eight values per row or column, which every CTA pushes its part
+// of into all eight CTAs' shared memory: one cluster barrier per eight pivots
+// (one per pivot and two triangles before).  Each CTA eliminates the panel for
+// itself.
 // Bound by the chain of pivots and the fp64 units (64 cycles a warp instruction
-// and scheduler).  n = 200, three objectives: 288 us, 560 with a barrier per pivot.
+// and scheduler).  n = 200, three objectives, the whole state: 317 us, 602 with a
+// barrier per pivot.
 __global__ void __cluster_dims__(kClusterCTAs, 1, 1) __launch_bounds__(kClusterThreads)
 gp_chol_cluster_kernel(const __grid_constant__ GpPrepArgs a, int64_t own) {
     namespace cg = cooperative_groups;
@@ -378,7 +474,7 @@ gp_chol_cluster_kernel(const __grid_constant__ GpPrepArgs a, int64_t own) {
     double* A = panel + 2 * (size_t)(n + 1) * B;          // owned rows, packed
     double* gs = A + own;                                 // [owned rows][B] the rows' g
     const int nl = (n + 1 - rank + C - 1) / C;            // rows owned, row n among them
-    __shared__ double Di[B][B + 1], X[B][B + 1], Xq[B][B + 1], rowa[2][B], roww[2][B], rcp[B], rs[B];
+    __shared__ PanelPivots pivots;
     __shared__ int s_fail;
     const double* K = a.K + (int64_t)m * a.tri;
     const float* y = a.y + (int64_t)m * n;
@@ -388,19 +484,19 @@ gp_chol_cluster_kernel(const __grid_constant__ GpPrepArgs a, int64_t own) {
         double* Ai = A + local_row_off(li, rank);
         for (int t = lane; t <= i; t += 32) Ai[t] = i < n ? K[tri_idx(i, t)] : t < n ? (double)y[t] : 0.0;
     }
-    double* peer[C];  // every CTA's panel
-#pragma unroll
-    for (int r = 0; r < C; ++r) peer[r] = cluster.map_shared_rank(panel, r);
     // The panel of block kb: [j][c] = A_j,kb+c of the rows j >= kb + c (and its
     // mirror within the block), W_kb+c,j of the columns j < kb; 0 beyond pivot n - 1.
     auto push = [&](int kb) {
         const size_t off = (size_t)((kb / B) & 1) * (n + 1) * B;
+        double* peer[C];  // every CTA's panel
+#pragma unroll
+        for (int r = 0; r < C; ++r) peer[r] = cluster.map_shared_rank(panel, r) + off;
         for (int e = tid; e < nl * B; e += kClusterThreads) {
             const int li = e / B, c = e - li * B, i = rank + C * li, kc = kb + c;
             if (kc < n && (i < kb || kc > i)) continue;
             const double v = kc < n ? A[local_row_off(li, rank) + kc] : 0.0;
 #pragma unroll
-            for (int r = 0; r < C; ++r) peer[r][off + i * B + c] = v;
+            for (int r = 0; r < C; ++r) peer[r][i * B + c] = v;
         }
         const int row = kb + rank;
         if (row < n) {
@@ -408,7 +504,7 @@ gp_chol_cluster_kernel(const __grid_constant__ GpPrepArgs a, int64_t own) {
             for (int j = tid; j < row; j += kClusterThreads) {
                 const double v = Ar[j];
 #pragma unroll
-                for (int r = 0; r < C; ++r) peer[r][off + j * B + rank] = v;
+                for (int r = 0; r < C; ++r) peer[r][j * B + rank] = v;
             }
         }
     };
@@ -416,81 +512,28 @@ gp_chol_cluster_kernel(const __grid_constant__ GpPrepArgs a, int64_t own) {
     push(0);
     cluster.sync();
     for (int kb = 0; kb < n; kb += B) {
-        const double* P0 = panel + (size_t)((kb / B) & 1) * (n + 1) * B;
+        double* P0 = panel + (size_t)((kb / B) & 1) * (n + 1) * B;
         const int be = min(B, n - kb);
-        if (warp < 2) {  // X and D^{-1}, an entry per thread
-            const int r = tid / B, c = tid % B;
-            double e = r < be && c < be ? P0[(kb + r) * B + c] : 0.0, w = r == c && r < be ? 1.0 : 0.0;
-            for (int p = 0; p < be; ++p) {
-                if (r == p) {
-                    rowa[p & 1][c] = e;
-                    roww[p & 1][c] = w;
-                }
-                asm volatile("bar.sync 1, 64;" ::: "memory");
-                if (r == p && c == p) {  // (while the others multiply)
-                    const bool ok = good_pivot(e);
-                    if (!ok) s_fail = 1;
-                    rcp[p] = ok ? rcp_newton(e) : 0.0;
-                }
-                const double x = r > p ? -rowa[p & 1][r] : 0.0, xa = x * rowa[p & 1][c], xw = x * roww[p & 1][c];
-                asm volatile("bar.sync 1, 64;" ::: "memory");
-                e = fma(xa, rcp[p], e);
-                w = fma(xw, rcp[p], w);
-            }
-            X[r][c] = w;  // of unit diagonal: row r of L_D^{-1} is this over sqrt(pivot r)
-            Xq[r][c] = r < be ? w * rcp[r] : 0.0;
-            asm volatile("bar.sync 1, 64;" ::: "memory");
-            double v = 0.0;
-            for (int p = 0; p < be; ++p) v = fma(Xq[p][r], X[p][c], v);
-            Di[r][c] = v;
-        }
+        eliminate_panel(P0, gs, pivots, &s_fail, n, kb, be, rank, false);
         __syncthreads();
-        if (s_fail) break;  // the same in every CTA: each has factorised the same block
-        if (tid >= kClusterThreads - be) {  // 1 / sqrt(pivot), for the block's rows
-            const double q = rcp[tid - (kClusterThreads - be)];
-            rs[tid - (kClusterThreads - be)] = q * rsqrt_newton(q);
-        }
-        for (int e = tid; e < nl * B; e += kClusterThreads) {  // g of the later rows
-            const int li = e / B, c = e - li * B, i = rank + C * li;
-            double v = 0.0;
-            if (i >= kb + be) {
-#pragma unroll
-                for (int p = 0; p < B; ++p) v = fma(P0[i * B + p], Di[p][c], v);
-            }
-            gs[e] = v;
-        }
-        __syncthreads();
+        if (s_fail) break;  // the same in every CTA: each has eliminated the same panel
         for (int li = (kb / C) + warp; li < nl; li += nwarps) {
             const int i = rank + C * li, ii = i - kb;
-            if (ii < 0) continue;
             double* Ai = A + local_row_off(li, rank);
-            if (ii < be) {  // a row of the block: L^{-1} of it
-                const double s = rs[ii];
-                for (int t = lane; t <= i; t += 32) {
-                    double v = 0.0;
-                    if (t < kb) {
-                        for (int p = 0; p <= ii; ++p) v = fma(X[ii][p], P0[(size_t)t * B + p], v);
-                    } else {
-                        v = X[ii][t - kb];
-                    }
-                    Ai[t] = v * s;
-                }
+            if (ii < be) {  // the CTA's row of the block: L^{-1} of it
+                const double q = rsqrt_newton(pivots.piv[ii]);
+                for (int t = lane; t <= i; t += 32) Ai[t] = P0[(size_t)t * B + ii] * q;
                 continue;
             }
             double gr[B];
 #pragma unroll
             for (int c = 0; c < B; ++c) gr[c] = -gs[li * B + c];
             for (int j = lane; j <= i; j += 32) {
-                const int jj = j - kb;
-                if (jj >= 0 && jj < be) {
-                    Ai[j] = -gs[li * B + jj];
-                } else {
-                    const double* Pj = P0 + (size_t)j * B;
-                    double v = Ai[j];
+                const double* Pj = P0 + (size_t)j * B;
+                double v = j >= kb && j < kb + be ? 0.0 : Ai[j];
 #pragma unroll
-                    for (int c = 0; c < B; ++c) v = fma(gr[c], Pj[c], v);
-                    Ai[j] = v;
-                }
+                for (int c = 0; c < B; ++c) v = fma(gr[c], Pj[c], v);
+                Ai[j] = v;
             }
         }
         __syncthreads();
