@@ -799,26 +799,34 @@ __global__ void __launch_bounds__(kMleThreads) gp_mle_kernel(const __grid_consta
 // runs at two lanes per clock per SM: an evaluation at n = 128 took 1.2 ms on one
 // SM.  Here CTA r owns rows i = r (mod 8) of the symmetric matrix, and K^{-1},
 // alpha and the determinant come from one elimination: the matrix is
-// augmented by row n, which holds y^T and 0, and its first n pivots are swept,
-//   A_kk <- -1 / A_kk,  A_ik <- A_ik / A_kk,  A_ij <- A_ij - A_ik A_kj / A_kk,
-// which leaves -K^{-1}, alpha^T = y^T K^{-1} in row n and -y^T K^{-1} y at its end
-// (n^3 / 2 multiply-adds, as many as a factor, its inverse and their product;
-// the pivots are the Cholesky factor's squared).  Pivots go in blocks of eight,
+// augmented by row n, which holds y^T and 0, and its first n pivots are swept in
+// place: before pivot t entry (i, t) is A_it, after it W_it, the elimination of the
+// identity, and after pivot i too what -K^{-1}_it has gathered, -sum_p W_pi W_pt / A_pp:
+// with the panel P and the multipliers g of eliminate_panel every entry takes
+//   A_ij -= g_i . P_j
+// (from 0 where i or j is a pivot of the block), which leaves -K^{-1}, -alpha^T in
+// row n and -y^T K^{-1} y at its end (n^3 / 2 multiply-adds, as many as a factor, its
+// inverse and their product; the pivots are the Cholesky factor's squared).  Pivots
+// go in blocks of eight,
 // so that a block costs one exchange: every CTA pushes its part of the next
-// block's columns into all eight CTAs' shared memory, and each inverts the
-// 8 x 8 block for itself.  The covariances and their slopes are kept for the
+// block's columns into all eight CTAs' shared memory, and each eliminates the
+// panel for itself.  The covariances and their slopes are kept for the
 // gradient where two CTAs still fit an SM (a GPU has room for 15 clusters of one
 // CTA per SM, a sixteenth would wait for them: the tuning loop has 8 starts of
 // two objectives).  An fp64 instruction holds a scheduler's unit for 64 cycles, so
 // what counts is their number: features are scaled once per evaluation,
 // categories and pivots compared as integers.
-// Measured (60 steps, 8 starts x 2 objectives, gp_mle_kernel against this): n = 64
-// 19.7 ms against 5.8, n = 128 72.8 against 17.6, n = 256 499 against 90; 64 fits at
-// n = 128 75.6 against 34.0, 128 fits 75.6 against 67.1.  Larger n than fits (about
-// 300) stay with gp_mle_kernel.  Keeping the squared differences as well cost the
-// second CTA per SM and was slower (25 ms at n = 128).
+// Measured (60 steps, 8 starts x 2 objectives, 4 or 8 parameters, gp_mle_kernel against
+// this): n = 64 19.7 ms against 5.9, n = 128 72.8 against 16.5, n = 256 471 against 78;
+// with one CTA per SM, n = 317 826 against 115 (covariances kept), n = 400 1608 against
+// 232, n = 500 2977 against 404.  64 fits at n = 128 75.6 against 32.2, 128 fits 75.6
+// against 63.4; 32 fits at n = 500 3051 against 606.  What does not fit (from 443
+// observations of 16 parameters, 519 of 2) stays with gp_mle_kernel.  Keeping the squared
+// differences as well cost the second CTA per SM and was slower (25 ms at n = 128).
+// The gradient's error against 64 bits is that of gp_mle_kernel (1.1e-13 at n = 128; a
+// sweep that multiplied by inverted blocks had 4.8e-13).
 constexpr int kMleB = kClusterB;
-constexpr int kMleClThreads = 256;
+constexpr int kMleClThreads = kClusterThreads;
 
 constexpr size_t kMleClTwo = 108 * 1024;  // shared memory of which two CTAs fit an SM
 
@@ -854,14 +862,16 @@ gp_mle_cluster_kernel(const __grid_constant__ MleArgs a, int64_t own, int keep) 
     double* gs = piv + n + 1;                             // [owned rows][B] a row's multipliers in an elimination step
     double* kvs = gs + (size_t)((n + 1 + C - 1) / C) * B;  // if kept: k / s_f^2 of the owned rows
     double* dks = kvs + own;                              // and its slope in r^2
-    __shared__ double th[kMleMaxP], g[kMleMaxP], il2[SCOOT_MAX_DIM], il[SCOOT_MAX_DIM];
+    __shared__ double th[kMleMaxP], g[kMleMaxP], am[2][kMleMaxP], il2[SCOOT_MAX_DIM], il[SCOOT_MAX_DIM];  // am: Adam's moments
     __shared__ double s_sf2, s_tau2, s_c1, s_c2, s_total;
     __shared__ double part[C][kMleMaxP + 1], red[nwarps][kMleMaxP + 1];
-    __shared__ double Dn[B][B + 1], rowb[2][B], rcp[2];
+    __shared__ PanelPivots pivots;
     __shared__ int s_fail;
     const int nl = (n + 1 - rank + C - 1) / C;  // owned rows, row n among them
-    double m1 = 0.0, m2 = 0.0;  // thread p: Adam's moments of parameter p
-    if (tid < P) th[tid] = a.theta0[(int64_t)sm * P + tid];
+    if (tid < P) {
+        th[tid] = a.theta0[(int64_t)sm * P + tid];
+        am[0][tid] = am[1][tid] = 0.0;
+    }
     if (tid == 0) s_fail = 0;
     // Term c of r^2 between rows i and k.
     auto term = [&](int c, int i, int k) {
@@ -881,20 +891,20 @@ gp_mle_cluster_kernel(const __grid_constant__ MleArgs a, int64_t own, int keep) 
         }
         return r2;
     };
-    double* peer[C];  // every CTA's panel
-#pragma unroll
-    for (int r = 0; r < C; ++r) peer[r] = cluster.map_shared_rank(panel, r);
     // The columns kb .. kb + 7 of the symmetric matrix into every CTA's panel,
     // [j][c] = A_j,kb+c (0 beyond the last pivot): an owned row j >= kb + c gives
     // its entries, the block's own rows those of the rows before them.
     auto push = [&](int kb) {
         const size_t off = (size_t)((kb / B) & 1) * (n + 1) * B;
+        double* peer[C];  // every CTA's panel
+#pragma unroll
+        for (int r = 0; r < C; ++r) peer[r] = cluster.map_shared_rank(panel, r) + off;
         for (int e = tid; e < nl * B; e += kMleClThreads) {
             const int li = e / B, c = e - li * B, i = rank + C * li, kc = kb + c;
             if (kc < n && kc > i) continue;
             const double v = kc < n ? A[local_row_off(li, rank) + kc] : 0.0;
 #pragma unroll
-            for (int r = 0; r < C; ++r) peer[r][off + i * B + c] = v;
+            for (int r = 0; r < C; ++r) peer[r][i * B + c] = v;
         }
         const int row = kb + rank;
         if (row < n) {
@@ -902,7 +912,7 @@ gp_mle_cluster_kernel(const __grid_constant__ MleArgs a, int64_t own, int keep) 
             for (int j = tid; j < row; j += kMleClThreads) {
                 const double v = Ar[j];
 #pragma unroll
-                for (int r = 0; r < C; ++r) peer[r][off + j * B + rank] = v;
+                for (int r = 0; r < C; ++r) peer[r][j * B + rank] = v;
             }
         }
     };
@@ -946,69 +956,34 @@ gp_mle_cluster_kernel(const __grid_constant__ MleArgs a, int64_t own, int keep) 
         push(0);
         cluster.sync();
         for (int kb = 0; kb < n; kb += B) {
-            const double* P0 = panel + (size_t)((kb / B) & 1) * (n + 1) * B;
+            double* P0 = panel + (size_t)((kb / B) & 1) * (n + 1) * B;
             const int be = min(B, n - kb);
-            if (warp < 2) {  // minus the inverse of the pivot block, an entry per thread
-                const int r = tid / B, c = tid % B;
-                double e = r < be && c < be ? P0[(kb + r) * B + c] : 0.0;
-                for (int p = 0; p < be; ++p) {
-                    if (r == p) rowb[p & 1][c] = e;
-                    asm volatile("bar.sync 1, 64;" ::: "memory");
-                    const double x = rowb[p & 1][r], y = rowb[p & 1][c];
-                    if (r == p && c == p) {  // (while the others multiply)
-                        piv[kb + p] = e;
-                        const bool ok = good_pivot(e);
-                        if (!ok) s_fail = 1;
-                        rcp[p & 1] = ok ? rcp_newton(e) : 0.0;
-                    }
-                    const double xy = r == p ? y : c == p ? x : -x * y;
-                    asm volatile("bar.sync 1, 64;" ::: "memory");
-                    const double q = rcp[p & 1];
-                    e = r == p ? (c == p ? -q : xy * q) : (c == p ? xy * q : fma(xy, q, e));
-                }
-                Dn[r][c] = r < be && c < be ? e : 0.0;
-            }
+            eliminate_panel(P0, gs, pivots, &s_fail, n, kb, be, rank, true);
             __syncthreads();
-            if (s_fail) break;  // the same in every CTA: each has swept the same block
-            for (int e = tid; e < nl * B; e += kMleClThreads) {  // the rows' multipliers
-                const int li = e / B, c = e - li * B, i = rank + C * li, ii = i - kb;
-                double v = 0.0;
-                if (ii >= 0 && ii < be) {
-                    v = -Dn[c][ii];
-                } else {
-#pragma unroll
-                    for (int p = 0; p < B; ++p) v = fma(P0[i * B + p], -Dn[p][c], v);
-                }
-                gs[e] = v;
-            }
-            __syncthreads();
+            if (s_fail) break;  // the same in every CTA: each has eliminated the same panel
+            if (tid < be) piv[kb + tid] = pivots.piv[tid];
             for (int li = warp; li < nl; li += nwarps) {
-                const int i = rank + C * li, ii = i - kb;
-                const bool pivot = ii >= 0 && ii < be;
+                const int i = rank + C * li;
+                const bool pivot = i >= kb && i < kb + be;
                 double* Ai = A + local_row_off(li, rank);
                 double gr[B];
 #pragma unroll
-                for (int c = 0; c < B; ++c) gr[c] = gs[li * B + c];
+                for (int c = 0; c < B; ++c) gr[c] = -gs[li * B + c];
                 for (int j = lane; j <= i; j += 32) {
-                    const int jj = j - kb;
-                    if (jj >= 0 && jj < be) {
-                        Ai[j] = pivot ? Dn[ii][jj] : gs[li * B + jj];
-                    } else {
-                        const double* Pj = P0 + (size_t)j * B;
-                        double v = pivot ? 0.0 : -Ai[j];
+                    const double* Pj = P0 + (size_t)j * B;
+                    double v = pivot || (j >= kb && j < kb + be) ? 0.0 : Ai[j];
 #pragma unroll
-                        for (int c = 0; c < B; ++c) v = fma(gr[c], Pj[c], v);
-                        Ai[j] = pivot ? v : -v;
-                    }
+                    for (int c = 0; c < B; ++c) v = fma(gr[c], Pj[c], v);
+                    Ai[j] = v;
                 }
             }
             __syncthreads();
             if (kb + B < n) {
                 push(kb + B);
-            } else if (n % C == rank) {  // row n: alpha and -y^T alpha, everywhere
+            } else if (n % C == rank) {  // row n: -alpha and -y^T alpha, everywhere
                 const double* Ar = A + local_row_off(n / C, rank);
                 for (int j = tid; j <= n; j += kMleClThreads)
-                    for (int r = 0; r < C; ++r) cluster.map_shared_rank(al, r)[j] = j < n ? Ar[j] : -Ar[j];
+                    for (int r = 0; r < C; ++r) cluster.map_shared_rank(al, r)[j] = -Ar[j];
             }
             cluster.sync();
         }
@@ -1073,8 +1048,8 @@ gp_mle_cluster_kernel(const __grid_constant__ MleArgs a, int64_t own, int keep) 
         }
         if (tid < P && ((a.free_mask >> tid) & 1u)) {  // projected Adam step on the free parameters
             const double step = a.lr * (1.0 - (double)it / a.steps), gp = g[tid];
-            m1 = 0.9 * m1 + 0.1 * gp;
-            m2 = 0.999 * m2 + 0.001 * gp * gp;
+            const double m1 = am[0][tid] = 0.9 * am[0][tid] + 0.1 * gp;
+            const double m2 = am[1][tid] = 0.999 * am[1][tid] + 0.001 * gp * gp;
             const double upd = step * (m1 / s_c1) / (sqrt(m2 / s_c2) + 1e-8);
             th[tid] = fmin(fmax(th[tid] + upd, a.lo[tid]), a.hi[tid]);
         }

@@ -83,6 +83,11 @@ def run(S, space, words, y, theta, kernel):
 @pytest.mark.parametrize("n,d,M,starts,kernel", [
     (1, 2, 1, 1, 0), (2, 3, 2, 3, 1), (7, 4, 1, 2, 0), (8, 4, 2, 2, 1), (9, 16, 1, 2, 0), (63, 5, 2, 2, 0), (64, 5, 1, 3, 1),
     (65, 5, 1, 2, 0), (136, 8, 4, 5, 0), (199, 16, 1, 2, 1), (200, 3, 1, 2, 0), (288, 4, 1, 1, 0), (640, 4, 1, 1, 1),
+    # the last and first n of each use of shared memory: two CTAs per SM, one that keeps the covariances, one that does
+    # not, the kernel of one block per fit
+    (212, 4, 1, 2, 1), (213, 4, 1, 1, 0), (317, 4, 1, 1, 0), (318, 4, 1, 1, 1), (325, 4, 1, 1, 0), (326, 4, 1, 1, 0),
+    (506, 4, 1, 1, 1), (507, 4, 1, 1, 0), (264, 16, 1, 1, 0), (265, 16, 1, 1, 1), (300, 16, 1, 1, 0), (301, 16, 1, 1, 0),
+    (442, 16, 1, 1, 0), (443, 16, 1, 1, 1),
 ])
 def test_evaluation(S, n, d, M, starts, kernel):
     space, words, u, y, theta = inputs(n, d, M, starts)
@@ -102,3 +107,23 @@ def test_not_positive_definite(S, n):
     _, lml, g = run(S, space, words, y, theta, 0)
     assert torch.isfinite(lml[0, 0]) and torch.isfinite(g[0]).all()
     assert lml[1, 0] == -math.inf and (g[1] == 0).all()
+
+
+@pytest.mark.parametrize("n,d", [(16, 3), (100, 5), (200, 4)])
+@pytest.mark.parametrize("noise", [1e-5, 1e-7])
+def test_repeated_observations(S, n, d, noise):
+    """Half of the observations repeat the other half and the noise is small: pivots of
+    the noise's size.  Bar, relative to the largest value: 8 n u / noise (u = 2^-53), the
+    rounding of a pivot of that size, twice, and of the n terms of each sum."""
+    space, words, u, y, theta = inputs(n, d, 2, 2)
+    order = np.argsort(Stream(n, "mle repeats").uniform(n))
+    for a in (words, u):
+        a[:, n // 2:] = a[:, :n - n // 2]
+        a[:] = a[:, order]
+    theta[..., d + 1] = math.log(noise)
+    _, lml, g = run(S, space, words, y, theta, 0)
+    want, wg = reference(words, u, y, theta, 0)
+    worst = max(float(((lml - want).abs() / want.abs()).max()),
+                float(((g - wg).abs() / wg.abs().amax(-1, keepdim=True)).max()))
+    print(f"mle repeated n={n} noise={noise}: {worst:.2e}")
+    assert worst <= 8 * n * 2.0 ** -53 / noise
