@@ -43,6 +43,17 @@
  *  - Objectives are maximised (Eq. 1 with the lambda signs applied).
  *  - A context is used by one host thread at a time.  Calls on one context
  *    that overlap on the GPU share its workspace: order them on one stream.
+ *  - Any scoring, selection or forest call on a context may use its workspace,
+ *    with or without a mask.  It grows when a call needs more than any call
+ *    before it, which waits for the device and cannot happen during stream
+ *    capture: make the largest call once before capturing.  A workspace
+ *    that a captured call has used is kept until the context is destroyed,
+ *    so its graph stays valid when a later call takes a larger one.
+ *    scoot_score_ehvi, scoot_score_ehvi_exact, unmasked scoot_rf_predict and,
+ *    above 256 observations, scoot_gp_posterior, scoot_score_ei and
+ *    scoot_score_mace go on without what they cannot have, by the kernels
+ *    that need none: captured on a context whose workspace is still too small
+ *    they may differ from the same call made eagerly in the last bits.
  */
 #ifndef SCOOT_H
 #define SCOOT_H

@@ -50,7 +50,7 @@ scoot_status scoot_compact(scoot_ctx* ctx, const uint8_t* mask, int64_t n, uint3
                            cudaStream_t st, ScootList* out, int fill_rows, int64_t fill_ld) {
     if (n > 0x7FFFFFFFll) return scoot_fail(ctx, SCOOT_EUNSUPPORTED, "compaction of %lld > 2^31 candidates", (long long)n);
     const size_t bytes = 256 + (size_t)n * sizeof(int32_t);
-    scoot_status s = scoot_workspace(ctx, bytes);
+    scoot_status s = scoot_workspace(ctx, bytes, st);
     if (s != SCOOT_OK) return s;
     out->count = static_cast<unsigned int*>(ctx->ws);
     out->list = reinterpret_cast<int32_t*>(static_cast<char*>(ctx->ws) + 256);

@@ -25,33 +25,65 @@ scoot_status scoot_enter(scoot_ctx* ctx) {
     return SCOOT_OK;
 }
 
-scoot_status scoot_workspace(scoot_ctx* ctx, size_t bytes) {
-    if (bytes <= ctx->ws_bytes) return SCOOT_OK;
+static bool is_capturing(void* st) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(static_cast<cudaStream_t>(st), &status) != cudaSuccess) {
+        cudaGetLastError();  // the legacy stream beside a capture, which it does not join
+        return false;
+    }
+    return status != cudaStreamCaptureStatusNone;
+}
+
+// A buffer of at least `bytes` in place of the current one, which queued kernels
+// may still read: freed once the device is idle, or kept, if a graph may read
+// it, until the context is destroyed.  Then the buffer doubles, so that what is kept
+// is less than what is in use.
+static bool replace_workspace(scoot_ctx* ctx, size_t bytes) {
     size_t want = bytes < (size_t(1) << 20) ? (size_t(1) << 20) : bytes;
-    if (ctx->ws) {
-        // The old buffer may still be read by queued kernels.
-        SCOOT_CUDA(ctx, cudaDeviceSynchronize());
-        SCOOT_CUDA(ctx, cudaFree(ctx->ws));
-        ctx->ws = nullptr;
-        ctx->ws_bytes = 0;
+    if (ctx->ws_in_graph && want < 2 * ctx->ws_bytes) want = 2 * ctx->ws_bytes;
+    void* p = nullptr;
+    if (cudaMalloc(&p, want) != cudaSuccess) {
+        cudaGetLastError();
+        if (want == bytes || cudaMalloc(&p, want = bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
     }
-    cudaError_t e = cudaMalloc(&ctx->ws, want);
-    if (e != cudaSuccess) {
-        ctx->ws = nullptr;
-        return scoot_fail(ctx, SCOOT_ENOMEM, "workspace of %zu bytes: %s", want, cudaGetErrorString(e));
+    if (ctx->ws_in_graph) {
+        ctx->ws_kept.push_back(ctx->ws);
+        ctx->ws_kept_bytes += ctx->ws_bytes;
+    } else if (ctx->ws) {
+        cudaDeviceSynchronize();
+        cudaFree(ctx->ws);
     }
+    ctx->ws = p;
     ctx->ws_bytes = want;
+    ctx->ws_in_graph = false;
+    return true;
+}
+
+scoot_status scoot_workspace(scoot_ctx* ctx, size_t bytes, void* st) {
+    const bool capture = is_capturing(st);
+    if (bytes > ctx->ws_bytes) {
+        if (ctx->ws && capture)
+            return scoot_fail(ctx, SCOOT_ECUDA, "a workspace of %zu bytes is needed and cannot grow during capture", bytes);
+        if (ctx->ws && !ctx->ws_in_graph) {  // gives its memory back first: the new one may need it
+            SCOOT_CUDA(ctx, cudaDeviceSynchronize());
+            SCOOT_CUDA(ctx, cudaFree(ctx->ws));
+            ctx->ws = nullptr;
+            ctx->ws_bytes = 0;
+        }
+        if (!replace_workspace(ctx, bytes)) return scoot_fail(ctx, SCOOT_ENOMEM, "no memory for a workspace of %zu bytes", bytes);
+    }
+    ctx->ws_in_graph |= capture;
     return SCOOT_OK;
 }
 
 bool scoot_workspace_try(scoot_ctx* ctx, size_t bytes, void* st) {
-    if (bytes <= ctx->ws_bytes) return true;
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(static_cast<cudaStream_t>(st), &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone &&
-        scoot_workspace(ctx, bytes) == SCOOT_OK)
-        return true;
-    cudaGetLastError();  // the caller goes on without it
-    return false;
+    const bool capture = is_capturing(st);
+    if (bytes > ctx->ws_bytes && (capture || !replace_workspace(ctx, bytes))) return false;
+    ctx->ws_in_graph |= capture;
+    return true;
 }
 
 static scoot_status record_event(scoot_ctx* ctx, void* st) {
@@ -124,6 +156,7 @@ scoot_status scoot_ctx_destroy(scoot_ctx* ctx) {
     cudaDeviceSynchronize();
     for (void* e : ctx->events) cudaEventDestroy(static_cast<cudaEvent_t>(e));
     if (ctx->ws) cudaFree(ctx->ws);
+    for (void* p : ctx->ws_kept) cudaFree(p);
     if (ctx->d_err) cudaFree(ctx->d_err);
     delete ctx;
     return SCOOT_OK;
@@ -185,7 +218,7 @@ scoot_status scoot_ctx_phase_times(scoot_ctx* ctx, int32_t cap, int32_t* h_kind,
 
 scoot_status scoot_ctx_workspace_bytes(const scoot_ctx* ctx, int64_t* bytes) {
     if (!ctx || !bytes) return SCOOT_EINVAL;
-    *bytes = (int64_t)ctx->ws_bytes;
+    *bytes = (int64_t)(ctx->ws_bytes + ctx->ws_kept_bytes);
     return SCOOT_OK;
 }
 

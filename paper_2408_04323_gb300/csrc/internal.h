@@ -25,6 +25,9 @@ struct scoot_ctx {
     std::string err;
     void* ws = nullptr;          // device workspace (grown on demand)
     size_t ws_bytes = 0;
+    bool ws_in_graph = false;    // a call being captured has used it
+    std::vector<void*> ws_kept;  // earlier ones that graphs may use, freed with the context
+    size_t ws_kept_bytes = 0;
     uint32_t* d_err = nullptr;   // device error word
     // Phase timing (scoot_ctx_set_timing): events recorded between the
     // launches of the last timed call, and the kind of each launch.
@@ -45,10 +48,12 @@ scoot_status scoot_fail(scoot_ctx* ctx, scoot_status s, const char* fmt, ...);
 void scoot_host_parallel(int count, const std::function<void(int)>& fn);
 // Make ctx->device current; sets an error on failure.
 scoot_status scoot_enter(scoot_ctx* ctx);
-// Ensure at least `bytes` of workspace (synchronising the device if it grows).
-scoot_status scoot_workspace(scoot_ctx* ctx, size_t bytes);
+// Ensure at least `bytes` of workspace for a call on stream st (synchronising the
+// device if it grows, unless a graph keeps the buffer it had).
+scoot_status scoot_workspace(scoot_ctx* ctx, size_t bytes, void* st);
 // Whether a call on stream st can have `bytes` of workspace; grows it if needed, but
-// not while st is being captured.  For routes with another that needs less.
+// not while st is being captured; what there is stays where it cannot.  For
+// routes with another that needs less.
 bool scoot_workspace_try(scoot_ctx* ctx, size_t bytes, void* st);
 
 static inline bool scoot_aligned16(const void* p) {

@@ -318,7 +318,7 @@ scoot_status scoot_select_pareto(scoot_ctx* ctx, const float* acq, int64_t lda, 
     if (n > 0 && !acq) return scoot_fail(ctx, SCOOT_EINVAL, "acq is NULL");
     if (n > 0 && lda < n) return scoot_fail(ctx, SCOOT_EINVAL, "lda = %lld < n", (long long)lda);
     if (front && front_cap < 0) return scoot_fail(ctx, SCOOT_EINVAL, "front_cap < 0");
-    if ((s = scoot_workspace(ctx, kWorkBytes)) != SCOOT_OK) return s;
+    if ((s = scoot_workspace(ctx, kWorkBytes, stream)) != SCOOT_OK) return s;
     char* ws = static_cast<char*>(ctx->ws);
     ParetoHead* head = reinterpret_cast<ParetoHead*>(ws);
     float4* samp = reinterpret_cast<float4*>(ws + kSampOffset);

@@ -719,7 +719,7 @@ scoot_status tc_direct(scoot_ctx* ctx, const ScoreArgs& a, const uint8_t* mask, 
     const size_t bytes = list_bytes + split_bytes + (groups ? (size_t)t.n_obj * a.n * 4 : 0);
     if (groups && !scoot_workspace_try(ctx, bytes, st)) return SCOOT_OK;
     *used = true;
-    scoot_status s = scoot_workspace(ctx, bytes);
+    scoot_status s = scoot_workspace(ctx, bytes, st);
     if (s != SCOOT_OK) return s;
     if (groups) t.sq = reinterpret_cast<float*>(static_cast<char*>(ctx->ws) + list_bytes + split_bytes);
     if (mask) {

@@ -134,7 +134,7 @@ scoot_status run(scoot_ctx* ctx, const float* acq, const uint8_t* mask, int64_t 
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     const int64_t slice = (n + blocks - 1) / blocks;
-    scoot_status s = scoot_workspace(ctx, (size_t)blocks * q * sizeof(uint64_t));
+    scoot_status s = scoot_workspace(ctx, (size_t)blocks * q * sizeof(uint64_t), st);
     if (s != SCOOT_OK) return s;
     uint64_t* partial = static_cast<uint64_t*>(ctx->ws);
     topq_pass1<QT><<<(unsigned)blocks, kTopqThreads, 0, st>>>(acq, mask, n, slice, q, partial);
