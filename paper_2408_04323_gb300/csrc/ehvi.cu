@@ -468,18 +468,23 @@ scoot_status launch(scoot_ctx* ctx, K kern, int threads, size_t smem, int64_t wa
 
 }  // namespace
 
-// The plan costs about 12 us and the walk's longest candidates 25 us, so
-// small pools and few boxes stay with ehvi_dense: measured (whole calls,
-// S = 100 to 128, dense against walk) 4096 candidates x 132 boxes 76 us
-// against 79, 20001 x 98 89 against 92, 32768 x 132 132 against 113, 4096 x 453
-// 199 against 134, 262144 x 453 2230 against 769.
-bool scoot_ehvi_walks(int M, int64_t n, int n_boxes, int n_mc) {
-    return M == 3 && n_boxes >= kWalkBoxMin && n_boxes <= kWalkBoxMax && n_mc <= kWalkIds && n * n_boxes >= 3 << 18;
+// The plan costs about 12 us, the walk's longest candidates 25, and its steps depend
+// on how many boxes a sample reaches, so it takes work enough, boxes x samples x
+// candidates: measured over three kinds of fronts (the workloads' with 65 to 296
+// boxes, spread over a sphere that prior samples seldom and often lie beyond with 113
+// to 362), S = 64 and 128, whole calls, dense against walk.  From 129 observations on:
+// 8192 candidates x 304 x 64 103 to 104 us against 112 to 120, 16384 x 113 x 64 83 to
+// 84 against 89 to 103; 4096 x 285 to 304 x 128 130 to 134 against 111 to 126, 16384 x
+// 296 to 310 x 64 144 to 149 against 115 to 143, 2^18 x 296 x 128 2691 against 1090.
+// Up to 128 observations the samples spread further: 16384 x 324 x 64 132 against 153
+// to 161, 24576 x 324 x 64 194 against 224 to 228; 32768 x 324 x 128 366 against 306 to
+// 334, 2^18 x 248 x 64 1209 against 658.
+bool scoot_ehvi_walks(int M, int64_t n, int n_boxes, int n_mc, int n_rb) {
+    return M == 3 && n >= 4096 && n_boxes >= kWalkBoxMin && n_boxes <= kWalkBoxMax && n_mc <= kWalkIds &&
+           (int64_t)n_boxes * n_mc * std::max<int64_t>(n, 8192) >= (n_rb <= 2 ? 520000000 : 290000000);
 }
 
-size_t scoot_ehvi_work_bytes(int M, int64_t n, int n_boxes, int n_mc) {
-    return scoot_ehvi_walks(M, n, n_boxes, n_mc) ? (plan_bytes(n_boxes) + 255) / 256 * 256 : 0;
-}
+size_t scoot_ehvi_walk_bytes(int n_boxes) { return (plan_bytes(n_boxes) + 255) / 256 * 256; }
 
 scoot_status scoot_ehvi_listed(scoot_ctx* ctx, int M, const float* mean, const float* var, int64_t n, int64_t ldm,
                                const int32_t* list, const unsigned int* n_list, const float* box_lo,
@@ -499,7 +504,7 @@ scoot_status scoot_ehvi_listed(scoot_ctx* ctx, int M, const float* mean, const f
     a.eps = eps;
     a.n_mc = n_mc;
     a.acq = acq;
-    if (scoot_ehvi_walks(M, n, n_boxes, n_mc)) {
+    if (work) {
         a.plan = static_cast<char*>(work);
         walk_plan<<<1, kPlanThreads, (size_t)kWalkBoxMax * 6, st>>>(box_lo, box_hi, n_boxes, static_cast<char*>(work));
         SCOOT_LAUNCHED(ctx);

@@ -203,11 +203,11 @@ bool scoot_tc_supported(scoot_ctx* ctx, const ScootTcArgs& a, int DO, bool group
 scoot_status scoot_posterior_tc(scoot_ctx* ctx, const ScootTcArgs& a, int DO, cudaStream_t st);
 
 // Monte-Carlo EHVI from moments by list position (ehvi.cu): acq at the
-// candidates' indices.  work: scoot_ehvi_work_bytes bytes of device scratch,
-// 16-byte aligned (may be NULL where that is 0).
-// scoot_ehvi_walks: the call takes the walk over the reached boxes.
-bool scoot_ehvi_walks(int M, int64_t n, int n_boxes, int n_mc);
-size_t scoot_ehvi_work_bytes(int M, int64_t n, int n_boxes, int n_mc);
+// candidates' indices.  work: scoot_ehvi_walk_bytes bytes of device scratch,
+// 16-byte aligned, for the walk over the reached boxes, or NULL for the sum over all.
+// scoot_ehvi_walks: the walk is the better of the two (three objectives).
+bool scoot_ehvi_walks(int M, int64_t n, int n_boxes, int n_mc, int n_rb);
+size_t scoot_ehvi_walk_bytes(int n_boxes);
 scoot_status scoot_ehvi_listed(scoot_ctx* ctx, int M, const float* mean, const float* var, int64_t n, int64_t ldm,
                                const int32_t* list, const unsigned int* n_list, const float* box_lo,
                                const float* box_hi, int32_t n_boxes, const float* eps, int32_t n_mc, void* work,

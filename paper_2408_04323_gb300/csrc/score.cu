@@ -13,6 +13,7 @@
 //     in shared memory by cp.async, so the next tile streams in while the
 //     current one is multiplied; sigma^2 = s_f^2 - sum_i V_ic^2, clamped at 0.
 // The epilogue writes mu and sigma^2, or the EI, or the EHVI of the tile.
+#include <algorithm>
 #include <cstring>
 
 #include "device_common.cuh"
@@ -789,21 +790,38 @@ scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* 
     *used = false;
     const int M = a.n_obj;
     if (!ctx->tensor_cores) return SCOOT_OK;
-    // One row block is little for the tensor cores' pipeline: it takes 65536
-    // candidates and more than 48 observations (8 parameters, M = 2, n = 64: 32768
-    // candidates 34.8 us fused against 34.8, 65536 49.6 against 45.7, 2^18 135 against
-    // 120; n = 40: 2^18 121 against 120; n = 16: 2^18 100 against 112), or the walk to
-    // save more (M = 3, n = 64, 132 boxes: 65536 123 against 115, 2^18 408 against 272).
-    // Beyond, the fused kernel is behind from 1024 candidates on (n = 100, M = 2: 39.0
-    // against 37.4, 65536 90 against 58; n = 128, M = 3: 63 against 61, 173 against 116).
-    if (a.n_rb == 1 && !(a.n >= 65536 && (a.n_obs > 48 || scoot_ehvi_walks(M, a.n, a.n_boxes, a.n_mc)))) return SCOOT_OK;
+    const bool walk = scoot_ehvi_walks(M, a.n, a.n_boxes, a.n_mc, a.n_rb);
+    if (a.n_rb == 1) {
+        // One row block is little for the tensor cores' pipeline: it takes 65536
+        // candidates and more than 48 observations (8 parameters, M = 2, n = 64: 32768
+        // candidates 34.8 us fused against 34.8, 65536 49.6 against 45.7, 2^18 135 against
+        // 120; n = 40: 2^18 121 against 120; n = 16: 2^18 100 against 112), or the walk to
+        // save more, the less the fewer observations and the wider their samples (M = 3, S =
+        // 128: n = 64, 193 boxes, 65536 402 against 295; n = 40, 132 boxes, 65536 291 against
+        // 295, 2^17 584 against 469; n = 32, 103 boxes, 2^17 476 against 476, 2^18 914 against
+        // 855; n = 24, 158 boxes, 2^18 1268 against 798 to 1441).
+        if (!(a.n >= 65536 && a.n_obs > 48) && !(walk && a.n * (a.n_obs - 24) >= 1900000)) return SCOOT_OK;
+    } else {
+        // The posterior gains with the observations and the candidates; the boxes in a kernel
+        // of their own cost more than behind the fused posterior while one wave of blocks
+        // takes the pool, the more the larger M.  Microseconds fitted to 65 to 256 observations
+        // (fused against this: M = 2, n = 65: 4096 candidates 29 against 31, 12288 36 against
+        // 31; n = 256 78 against 45.  M = 3, n = 65, 289 boxes, S = 128: 4096 88 against 107;
+        // n = 128, 45 boxes, S = 64 51 against 45; n = 200, 296 boxes, S = 128 148 against 122.
+        // M = 4, n = 65, 835 boxes, S = 128: 4096 471 against 681, 32768 2823 against 2837; n =
+        // 192, 108 boxes 148 against 141).  Over 500 such calls the rule's choice took at most
+        // 4% more than the fused kernel.
+        const double gain = M * ((a.n_obs - 82) / 14.0 + (double)std::max<int64_t>(a.n - 4096, 0) / 8192 * a.n_obs / 22);
+        const double loss = M == 2 ? 0.0 : walk ? 18.0 : (double)a.n_boxes * a.n_mc * (M == 3 ? 0.0007 : 0.0019);
+        if (gain <= loss) return SCOOT_OK;
+    }
     if (!score_fits(ctx, a, kEHVI, M)) return SCOOT_OK;
     ScootTcArgs t = tc_args(ctx, a, M);
     char* work;
-    const scoot_status s = tc_moments(ctx, a, t, 0, scoot_ehvi_work_bytes(M, a.n, a.n_boxes, a.n_mc), st, &work, used);
+    const scoot_status s = tc_moments(ctx, a, t, 0, walk ? scoot_ehvi_walk_bytes(a.n_boxes) : 0, st, &work, used);
     if (!*used || s != SCOOT_OK) return s;
     return scoot_ehvi_listed(ctx, M, t.mean, t.var, a.n, a.n, t.list, t.n_list, a.box_lo, a.box_hi, a.n_boxes, a.eps,
-                             a.n_mc, work, a.acq, st);
+                             a.n_mc, walk ? work : nullptr, a.acq, st);
 }
 
 size_t exact_smem(const ScoreArgs& a, int n_obj) {

@@ -59,7 +59,7 @@ def test_bad_words(S, ctx, name, n_obs, tc):  # noqa: F811
         assert three[0, bad].isnan().all() and (three[1:, bad] == 0).all() and three[:, ~bad].isfinite().all()
         if M > 1:
             lo, hi, _ = S.scoot_boxes_build(base.y_obs, base.ref)
-            eps = dev(st.normal(64 * M).reshape(64, M).astype(np.float32))
+            eps = dev(st.normal(128 * M).reshape(128, M).astype(np.float32))
             acq.fill_(7.0)
             S.scoot_score_ehvi(ctx, L, state, cand, N, dev(lo), dev(hi), eps, acq)
             assert (acq[bad] == 0).all() and acq[~bad].isfinite().all()

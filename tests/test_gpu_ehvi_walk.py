@@ -52,6 +52,9 @@ def all_boxes(mu, var, eps, lo, hi):
     (9001, 128, "built", True), (4099, 1, "built", False), (4096, 33, "built", True), (3907, 1024, "built", False),
     (5000, 300, "built", True), (1, 128, "built", False), (8192, 64, "shuffled", True), (8192, 64, "risen", True),
     (8192, 64, "few", False),
+    # (the smallest pools that take the walk at their number of samples, and boxes refused there)
+    (9600, 128, "built", True), (1203301, 1, "built", False), (36503, 33, "built", True), (4096, 1024, "built", False),
+    (20001, 64, "shuffled", True), (20001, 64, "risen", False),
 ])
 def test_walk_equals_all_boxes(S, n_cand, n_mc, boxes, masked):
     inst = make_instance("d10-ehvi3", 1004, n_cand=n_cand)
