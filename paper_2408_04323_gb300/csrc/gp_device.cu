@@ -571,7 +571,7 @@ gp_chol_cluster_kernel(const __grid_constant__ GpPrepArgs a, int64_t own) {
 }
 
 constexpr int kMleMaxP = SCOOT_MAX_DIM + 2;  // ln l_1 .. ln l_d, ln s_f^2, ln tau^2
-constexpr int kMleNoScratchN = 128;           // no scratch up to this n (the cluster kernel's, and more, fits)
+constexpr int kMleNoScratchN = 128;           // no scratch up to this n: the matrices fit shared memory
 constexpr int kMleThreads = 512;
 
 struct MleArgs {
@@ -587,7 +587,7 @@ struct MleArgs {
     double* theta;                           // [S][M][P]
     double* lml;                             // [S][M]
     double* grad;                            // [S][M][P] or nullptr
-    double* scratch;                         // [S M][2][tri] when n > kMleNoScratchN
+    double* scratch;                         // [S M][2][tri] when n > kMleNoScratchN (else in shared memory)
 };
 
 // Features of the observations, once per call: one thread per (j, c).
@@ -626,7 +626,7 @@ __device__ __forceinline__ void matern_slope(double r2, int kernel, double* k, d
     }
 }
 
-// (For more observations than gp_mle_cluster_kernel holds.)
+// (For more observations than gp_mle_cluster_kernel holds, and for many fits of few.)
 // One block per (start s, objective m): `steps` projected Adam steps on the
 // log marginal likelihood (beta1 0.9, beta2 0.999, eps 1e-8, step size
 // lr (1 - t / steps)), then the likelihood and gradient at the result.  Each
@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(kMleThreads) gp_mle_kernel(const __grid_consta
     double* al = z + n;                                  // [n] alpha
     double* col = al + n;                                // [2][n]
     double* U = col + 2 * n;                             // [d][n]: feature c of observation j at c n + j
-    double* A = a.scratch + (size_t)sm * 2 * a.tri;
+    double* A = a.scratch ? a.scratch + (size_t)sm * 2 * a.tri : U + (size_t)n * d;
     double* W = A + a.tri;
     __shared__ double th[kMleMaxP], m1[kMleMaxP], m2[kMleMaxP], g[kMleMaxP];
     __shared__ double il2[SCOOT_MAX_DIM];  // 1 / l_c^2
@@ -1281,7 +1281,17 @@ scoot_status scoot_gp_mle(scoot_ctx* ctx, const scoot_param* h_space, int32_t d,
     int optin = 0;
     SCOOT_CUDA(ctx, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
     const MleClSizes cl = mle_cl_sizes(n, d);
-    if (cl.bytes + 8192 <= (size_t)optin) {
+    // Eight CTAs per fit share its pivot rows' work but each runs their chain, so where
+    // the fits alone fill the SMs, a block each, a wave of blocks ends before the clusters
+    // do: those get 80 + 0.6 n fits done in its time on 152 SMs.  (60 steps, n = 16: 64 fits
+    // 3.7 ms against 4.2 by blocks, 128 7.2 against 4.2; n = 32: 128 fits 10.2 against 7.4; n =
+    // 64: 64 fits 10.6 against 18.7, 128 20.9 against 18.7, 512 77.8 against 74.6; n = 128: 512
+    // fits 229 against 278.)
+    int sms = 0;
+    SCOOT_CUDA(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
+    const int fits = n_starts * n_obj, waves = (fits + sms - 1) / sms;
+    const bool blocks = n <= kMleNoScratchN && fits * 152.0 > (double)waves * sms * (80.0 + 0.6 * n);
+    if (!blocks && cl.bytes + 8192 <= (size_t)optin) {
         const int keep = cl.bytes + cl.keep_bytes <= kMleClTwo || (cl.bytes > kMleClTwo && cl.bytes + cl.keep_bytes + 8192 <= (size_t)optin);
         const size_t bytes = cl.bytes + (keep ? cl.keep_bytes : 0);
         SCOOT_CUDA(ctx, cudaFuncSetAttribute(gp_mle_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
@@ -1289,8 +1299,7 @@ scoot_status scoot_gp_mle(scoot_ctx* ctx, const scoot_param* h_space, int32_t d,
         SCOOT_LAUNCHED(ctx);
         return SCOOT_OK;
     }
-    if (!a.scratch) return scoot_fail(ctx, SCOOT_EUNSUPPORTED, "shared memory of %d bytes is too small", optin);
-    const size_t smem = (size_t)(7 * n + (size_t)n * d) * sizeof(double);
+    const size_t smem = (size_t)(7 * n + (size_t)n * d) * sizeof(double) + (a.scratch ? 0 : (size_t)2 * a.tri * sizeof(double));
     SCOOT_CUDA(ctx, cudaFuncSetAttribute(gp_mle_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     gp_mle_kernel<<<n_starts * n_obj, kMleThreads, smem, st>>>(a);
     SCOOT_LAUNCHED(ctx);

@@ -88,6 +88,8 @@ def run(S, space, words, y, theta, kernel):
     (212, 4, 1, 2, 1), (213, 4, 1, 1, 0), (317, 4, 1, 1, 0), (318, 4, 1, 1, 1), (325, 4, 1, 1, 0), (326, 4, 1, 1, 0),
     (506, 4, 1, 1, 1), (507, 4, 1, 1, 0), (264, 16, 1, 1, 0), (265, 16, 1, 1, 1), (300, 16, 1, 1, 0), (301, 16, 1, 1, 0),
     (442, 16, 1, 1, 0), (443, 16, 1, 1, 1),
+    # enough fits of few observations for a block each, with the matrices in shared memory
+    (1, 2, 2, 64, 0), (17, 5, 2, 64, 1), (64, 4, 1, 152, 0), (100, 16, 1, 152, 0), (110, 3, 1, 152, 1),
 ])
 def test_evaluation(S, n, d, M, starts, kernel):
     space, words, u, y, theta = inputs(n, d, M, starts)
