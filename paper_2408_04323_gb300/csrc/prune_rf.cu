@@ -130,6 +130,7 @@ struct RfArgs {
     const int32_t* list;          // live candidates (NULL: all of 0 .. n-1)
     const unsigned int* n_list;
     int32_t max_chunk_nodes;
+    int64_t rank_from;            // rf_ranked_kernel takes lists from this length on, rf_kernel<true> shorter ones
 };
 
 // Persistent blocks of 256 threads score tiles of 32 candidates: lane l of
@@ -141,6 +142,8 @@ struct RfArgs {
 // feature values sit in shared memory as feat[f][slot], so that a lane's reads
 // stay in its own bank whatever features the lanes ask for.  The eight partial
 // vote counts of a candidate are added through shared memory.
+// kShort: the call may be rf_ranked_kernel's (see rank_from).
+template <bool kShort>
 __global__ void __launch_bounds__(kRfThreads)
 rf_kernel(const __grid_constant__ RfArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -155,6 +158,7 @@ rf_kernel(const __grid_constant__ RfArgs a) {
     const int tid = threadIdx.x;
     const int slot = tid & (kRfCand - 1), grp = tid / kRfCand;
     const int64_t n_work = a.list ? (int64_t)*a.n_list : a.n;
+    if (kShort && n_work >= a.rank_from) return;
     const int64_t n_tiles = (n_work + kRfCand - 1) / kRfCand;
     uint32_t feasible = 0;
 
@@ -269,6 +273,7 @@ constexpr int kRankVotes = 32767;         // votes of a leaf
 constexpr uint32_t kRankEnd = 8191u << 19;
 constexpr int kRankThreads = 1024;
 constexpr int64_t kRankFrom = 400000000;  // candidates x trees x depth that pay for the ranking
+constexpr int64_t kRankShallow = 160;     // trees x levels beyond two that do
 constexpr int kRankTiles = 4;             // tiles of 32 candidates per block, eight groups of trees each
 constexpr int kRankWalkThreads = kRankTiles * kRfThreads;
 
@@ -279,6 +284,8 @@ struct RankArgs {
     uint2* nodes;      // [n_nodes] ranked nodes, with the child's number for its address
     float* thr;        // [d][kRankThr] distinct thresholds, increasing
     int32_t* n_thr;    // [d]
+    const unsigned int* n_list;  // live candidates (NULL: all), and the fewest that pay for the ranking
+    int64_t rank_from;
 };
 
 // Block f: the distinct thresholds of feature f, sorted, and the ranked nodes
@@ -287,6 +294,7 @@ __global__ void __launch_bounds__(kRankThreads) rank_forest_kernel(const __grid_
     __shared__ float key[kRankThr];
     __shared__ int s_cnt, s_wt[kRankThreads / 32];
     const int f = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (a.n_list && (int64_t)*a.n_list < a.rank_from) return;
     const uint2* nodes = reinterpret_cast<const uint2*>(a.forest + a.off_nodes);
     const int4* chunks = reinterpret_cast<const int4*>(a.forest + a.off_chunks);  // .z first node, .w nodes
     if (tid == 0) s_cnt = 0;
@@ -387,6 +395,7 @@ rf_ranked_kernel(const __grid_constant__ RfArgs a, const uint2* __restrict__ nod
     const int half = warp % kRankTiles, grp = warp / kRankTiles;
     const uint32_t node0 = (uint32_t)__cvta_generic_to_shared(snodes);
     const int64_t n_work = a.list ? (int64_t)*a.n_list : a.n;
+    if (n_work < a.rank_from) return;
     const int64_t n_tiles = (n_work + kRfCand - 1) / kRfCand, step_tiles = (int64_t)gridDim.x * kRankTiles;
     const int64_t tile0 = (int64_t)blockIdx.x * kRankTiles;
     if (tile0 < n_tiles) {
@@ -564,11 +573,18 @@ scoot_status scoot_rf_predict(scoot_ctx* ctx, const scoot_forest_layout* L, cons
     // against this (100 trees of 1800 nodes in all; 100 of 3300; 200 of 12100): 2^17 candidates 54 us
     // against 52, 63 against 64, 161 against 155; 2^18 97 against 88, 112 against 107, 299 against 263;
     // 2^20 380 against 289, 439 against 353, 1180 against 894; 2^22 4967 against 3479.
-    // With a mask about half of the pool is walked.
+    // A candidate's features are ranked too, which shallow trees do not pay for (2^22
+    // candidates, 12 parameters: 40 trees of depth 2 388 against 529, of depth 4 435 against
+    // 525; 100 of depth 3 865 against 906, of depth 4 1187 against 971).
+    // How many candidates a mask leaves the device alone knows: where half of the pool would
+    // pay, both walks are launched, and one of them returns (2^20 candidates, 200 trees, 2% of
+    // them live: rf_kernel alone 68 us, so 76, with the ranking done for them 91).
     const size_t list_bytes = mask ? ((256 + (size_t)n * 4 + 255) & ~(size_t)255) : 0;
     const size_t node_bytes = ((size_t)L->n_nodes * 8 + 255) & ~(size_t)255;
-    const bool ranked = L->n_nodes <= kRankNodes && L->leaf_scale <= kRankVotes &&
-                        n * L->n_trees * (L->max_depth + 1) >= (mask ? kRankFrom * 2 : kRankFrom) &&
+    const int64_t visits = (int64_t)L->n_trees * (L->max_depth + 1), rank_from = (kRankFrom + visits - 1) / visits;
+    const bool ranked = L->n_nodes <= kRankNodes && L->leaf_scale <= kRankVotes && L->max_depth >= 3 &&
+                        (int64_t)L->n_trees * (L->max_depth - 2) >= kRankShallow &&
+                        n >= (mask ? 2 * rank_from : rank_from) &&
                         scoot_workspace_try(ctx, list_bytes + node_bytes + (size_t)L->d * kRankThr * 4 + 256, st);
     if (mask) {
         // Walk only the candidates still in play; the others get 0 votes.
@@ -578,6 +594,7 @@ scoot_status scoot_rf_predict(scoot_ctx* ctx, const scoot_forest_layout* L, cons
         a.n_list = lst.count;
     }
     if (ranked) {
+        a.rank_from = rank_from;
         char* ws = static_cast<char*>(ctx->ws) + list_bytes;
         RankArgs r;
         r.forest = a.forest;
@@ -588,6 +605,8 @@ scoot_status scoot_rf_predict(scoot_ctx* ctx, const scoot_forest_layout* L, cons
         r.nodes = reinterpret_cast<uint2*>(ws);
         r.thr = reinterpret_cast<float*>(ws + node_bytes);
         r.n_thr = reinterpret_cast<int32_t*>(ws + node_bytes + (size_t)L->d * kRankThr * 4);
+        r.n_list = a.n_list;
+        r.rank_from = rank_from;
         rank_forest_kernel<<<(unsigned)L->d, kRankThreads, 0, st>>>(r);
         SCOOT_LAUNCHED(ctx);
         const size_t rsmem = (size_t)kRankTiles * 16 * kRfCand * 4 + (size_t)kRfGroups * kRankTiles * kRfCand * 4 +
@@ -601,19 +620,20 @@ scoot_status scoot_rf_predict(scoot_ctx* ctx, const scoot_forest_layout* L, cons
                                                (n + kRankTiles * kRfCand - 1) / (kRankTiles * kRfCand));
         kern<<<(unsigned)grid, kRankWalkThreads, rsmem, st>>>(a, r.nodes, r.thr, r.n_thr, L->n_nodes);
         SCOOT_LAUNCHED(ctx);
-        return SCOOT_OK;
+        if (!mask) return SCOOT_OK;
     }
     a.max_chunk_nodes = max_chunk_nodes;
     const size_t smem = (size_t)max_chunk_nodes * 8 + (size_t)kRfCand * L->d * 4 +
                         (size_t)kRfGroups * kRfCand * 4 + (size_t)L->n_trees * 4;
-    SCOOT_CUDA(ctx, cudaFuncSetAttribute(rf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    auto kern = ranked ? rf_kernel<true> : rf_kernel<false>;
+    SCOOT_CUDA(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    SCOOT_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rf_kernel, kRfThreads, smem));
+    SCOOT_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kRfThreads, smem));
     if (per_sm < 1) return scoot_fail(ctx, SCOOT_EUNSUPPORTED, "forest chunk does not fit in shared memory");
     const int64_t tiles = (n + kRfCand - 1) / kRfCand;
     int64_t blocks = (int64_t)sm_count(ctx->device) * per_sm;
     if (blocks > tiles) blocks = tiles;
-    rf_kernel<<<(unsigned)blocks, kRfThreads, smem, st>>>(a);
+    kern<<<(unsigned)blocks, kRfThreads, smem, st>>>(a);
     SCOOT_LAUNCHED(ctx);
     return SCOOT_OK;
 }

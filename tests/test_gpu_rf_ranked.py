@@ -83,3 +83,44 @@ def test_ranked_walk_equals_float_walk(S, n, d, trees, size, distinct, chain):
     assert torch.equal(votes.long(), torch.where(live, want, 0))
     ok = live & (2 * want >= 255 * trees)
     assert torch.equal(mask.bool(), ok) and int(count.item()) == int(ok.sum())
+
+
+@pytest.mark.parametrize("size,depth", [(255, 7), (13, 3)])
+def test_both_sides_of_the_shortest_list(S, size, depth):
+    """A masked call leaves the choice of the walk to the device: one live candidate
+    fewer than the ranked walk takes, as many, none and all give the votes of the
+    unmasked walk of a small pool."""
+    n, d, trees = 1 << 20, 6, 180
+    st = Stream(size, "ranked lists")
+    grid = st.normal(50).astype(np.float32)
+    parts = [tree(st, d, size, grid, False) for _ in range(trees)]
+    offs = np.arange(trees + 1, dtype=np.int32) * size
+    if size * trees > 16380:  # within the ranked walk's nodes
+        keep = 16380 // size
+        parts, offs, trees = parts[:keep], offs[:keep + 1], keep
+    nodes = np.concatenate(parts)
+    space = np.zeros(d, PARAM)
+    space["kind"], space["lo"], space["hi"] = CONTINUOUS, -10, 10
+    L = S.scoot_forest_layout_init(nodes, offs, d, 255)
+    assert L.max_depth >= depth
+    blob = torch.from_numpy(S.scoot_forest_pack(L, nodes, offs)).cuda()
+    cand = torch.from_numpy(st.normal(d * n).reshape(d, n).astype(np.float32).view(np.int32)).cuda()
+    edge = -(-400000000 // (trees * (L.max_depth + 1)))
+    want = torch.empty(n, dtype=torch.int32, device="cuda")
+    with S.Context(0) as ctx:
+        for at in range(0, n, 1 << 16):  # pools that are not ranked
+            S.scoot_rf_predict(ctx, L, blob, space, cand[:, at:at + (1 << 16)].contiguous(), 1 << 16, 1, 2,
+                               want[at:at + (1 << 16)])
+        order = torch.randperm(n, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+        for live in (0, 1, edge - 1, edge, n):
+            assert live <= n
+            mask0 = torch.zeros(n, dtype=torch.uint8, device="cuda")
+            mask0[order[:live]] = 1
+            mask, votes = mask0.clone(), torch.full((n,), -1, dtype=torch.int32, device="cuda")
+            count = torch.zeros(1, dtype=torch.int64, device="cuda")
+            S.scoot_rf_predict(ctx, L, blob, space, cand, n, 1, 2, votes, mask, count)
+            ctx.check()
+            on = mask0.bool()
+            assert torch.equal(votes, torch.where(on, want, 0))
+            ok = on & (2 * want.long() >= 255 * trees)
+            assert torch.equal(mask.bool(), ok) and int(count.item()) == int(ok.sum())
