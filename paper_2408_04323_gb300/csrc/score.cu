@@ -790,7 +790,8 @@ scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* 
     *used = false;
     const int M = a.n_obj;
     if (!ctx->tensor_cores) return SCOOT_OK;
-    const bool walk = scoot_ehvi_walks(M, a.n, a.n_boxes, a.n_mc, a.n_rb);
+    const int64_t live = a.mask ? a.n / 2 : a.n;  // (about what the constraints and the forest leave)
+    const bool walk = scoot_ehvi_walks(M, live, a.n_boxes, a.n_mc, a.n_rb);
     if (a.n_rb == 1) {
         // One row block is little for the tensor cores' pipeline: it takes 65536
         // candidates and more than 48 observations (8 parameters, M = 2, n = 64: 32768
@@ -800,7 +801,7 @@ scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* 
         // 128: n = 64, 193 boxes, 65536 402 against 295; n = 40, 132 boxes, 65536 291 against
         // 295, 2^17 584 against 469; n = 32, 103 boxes, 2^17 476 against 476, 2^18 914 against
         // 855; n = 24, 158 boxes, 2^18 1268 against 798 to 1441).
-        if (!(a.n >= 65536 && a.n_obs > 48) && !(walk && a.n * (a.n_obs - 24) >= 1900000)) return SCOOT_OK;
+        if (!(a.n >= 65536 && a.n_obs > 48) && !(walk && live * (a.n_obs - 24) >= 1900000)) return SCOOT_OK;
     } else {
         // The posterior gains with the observations and the candidates; the boxes in a kernel
         // of their own cost more than behind the fused posterior while one wave of blocks
@@ -811,7 +812,7 @@ scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* 
         // M = 4, n = 65, 835 boxes, S = 128: 4096 471 against 681, 32768 2823 against 2837; n =
         // 192, 108 boxes 148 against 141).  Over 500 such calls the rule's choice took at most
         // 4% more than the fused kernel.
-        const double gain = M * ((a.n_obs - 82) / 14.0 + (double)std::max<int64_t>(a.n - 4096, 0) / 8192 * a.n_obs / 22);
+        const double gain = M * ((a.n_obs - 82) / 14.0 + (double)std::max<int64_t>(live - 4096, 0) / 8192 * a.n_obs / 22);
         const double loss = M == 2 ? 0.0 : walk ? 18.0 : (double)a.n_boxes * a.n_mc * (M == 3 ? 0.0007 : 0.0019);
         if (gain <= loss) return SCOOT_OK;
     }
