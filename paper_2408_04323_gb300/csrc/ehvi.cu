@@ -474,14 +474,15 @@ scoot_status launch(scoot_ctx* ctx, K kern, int threads, size_t smem, int64_t wa
 // boxes, spread over a sphere that prior samples seldom and often lie beyond with 113
 // to 362), S = 64 and 128, whole calls, dense against walk.  From 129 observations on:
 // 8192 candidates x 304 x 64 103 to 104 us against 112 to 120, 16384 x 113 x 64 83 to
-// 84 against 89 to 103; 4096 x 285 to 304 x 128 130 to 134 against 111 to 126, 16384 x
+// 84 against 89 to 103; 4096 x 285 to 304 x 128 130 to 134 against 111 to 126 (2300 x 452 x
+// 100 142 fused against 103), 16384 x
 // 296 to 310 x 64 144 to 149 against 115 to 143, 2^18 x 296 x 128 2691 against 1090.
 // Up to 128 observations the samples spread further: 16384 x 324 x 64 132 against 153
 // to 161, 24576 x 324 x 64 194 against 224 to 228; 32768 x 324 x 128 366 against 306 to
 // 334, 2^18 x 248 x 64 1209 against 658.
 bool scoot_ehvi_walks(int M, int64_t n, int n_boxes, int n_mc, int n_rb) {
-    return M == 3 && n >= 4096 && n_boxes >= kWalkBoxMin && n_boxes <= kWalkBoxMax && n_mc <= kWalkIds &&
-           (int64_t)n_boxes * n_mc * std::max<int64_t>(n, 8192) >= (n_rb <= 2 ? 520000000 : 290000000);
+    return M == 3 && n * n_boxes >= 3 << 18 && n_boxes >= kWalkBoxMin && n_boxes <= kWalkBoxMax && n_mc <= kWalkIds &&
+           (int64_t)n_boxes * n_mc * std::max<int64_t>(n, 8192) >= (n_rb <= 2 ? 520000000 : 230000000);
 }
 
 size_t scoot_ehvi_walk_bytes(int n_boxes) { return (plan_bytes(n_boxes) + 255) / 256 * 256; }

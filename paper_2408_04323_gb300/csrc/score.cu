@@ -808,12 +808,18 @@ scoot_status tc_ehvi(scoot_ctx* ctx, const ScoreArgs& a, cudaStream_t st, bool* 
         // takes the pool, the more the larger M.  Microseconds fitted to 65 to 256 observations
         // (fused against this: M = 2, n = 65: 4096 candidates 29 against 31, 12288 36 against
         // 31; n = 256 78 against 45.  M = 3, n = 65, 289 boxes, S = 128: 4096 88 against 107;
-        // n = 128, 45 boxes, S = 64 51 against 45; n = 200, 296 boxes, S = 128 148 against 122.
+        // n = 128, 45 boxes, S = 64 51 against 45; n = 200, 296 boxes, S = 128 148 against 122; the
+        // walk, n = 129, S = 128: 303 boxes 115 against 146, 452 142 against 116.
         // M = 4, n = 65, 835 boxes, S = 128: 4096 471 against 681, 32768 2823 against 2837; n =
-        // 192, 108 boxes 148 against 141).  Over 500 such calls the rule's choice took at most
-        // 4% more than the fused kernel.
-        const double gain = M * ((a.n_obs - 82) / 14.0 + (double)std::max<int64_t>(live - 4096, 0) / 8192 * a.n_obs / 22);
-        const double loss = M == 2 ? 0.0 : walk ? 18.0 : (double)a.n_boxes * a.n_mc * (M == 3 ? 0.0007 : 0.0019);
+        // 192, 108 boxes 148 against 141).  Over 700 such calls the rule's choice took at most 5%
+        // more than the fused kernel, but where most samples lie beyond a front of 300 boxes
+        // the walk visits many: n = 128 to 160, S = 128, 8192 to 16384 candidates 158 against 164
+        // to 222 against 270.
+        const double gain = M * ((a.n_obs - (a.n_rb >= 4 ? 62 : 82)) / 14.0 + (double)std::max<int64_t>(live - 4096, 0) / 8192 * a.n_obs / 22);
+        // (Summing all boxes takes 32 samples at a time; a walk takes those there are.)
+        const double work = (double)a.n_boxes * a.n_mc, all = (double)a.n_boxes * ((a.n_mc + 31) / 32 * 32);
+        const double loss = M == 2 ? 0.0 : walk ? 18.0 - 0.0012 * (std::max(all - 36000, 0.0) + all - work)
+                                               : work * (M == 3 ? 0.0007 : 0.0019);
         if (gain <= loss) return SCOOT_OK;
     }
     if (!score_fits(ctx, a, kEHVI, M)) return SCOOT_OK;
