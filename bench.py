@@ -47,8 +47,8 @@ FP32_LANES_PER_SM = 128
 # keyed by (kernel, workload), valid only while the kernel's sources are
 # unchanged (sha256 prefix of their contents when the counters were taken).
 KERNEL_FILES = {"prune": ["prune_rf.cu"], "rf": ["prune_rf.cu"],
-                "score": ["score.cu", "posterior_tc.cu", "device_common.cuh"],
-                "posterior": ["posterior_tc.cu", "device_common.cuh"], "fant_pass": ["fantasy.cu", "device_common.cuh"],
+                "score": ["score.cu", "posterior_tc.cu", "ehvi.cu", "approx.cuh", "device_common.cuh"],
+                "posterior": ["posterior_tc.cu", "approx.cuh", "device_common.cuh"], "fant_pass": ["fantasy.cu", "device_common.cuh"],
                 "topq": ["topq.cu", "device_common.cuh"], "pareto": ["pareto.cu"]}
 TRAFFIC = {
     # d12-fantasy: captured on a 2^20 pool of the same workload, scaled to the 2^22 launch by its

@@ -804,9 +804,15 @@ scoot_status scoot_select_topq_static(const float* acq, const uint8_t* mask, int
  * `steps` dependent steps through a binary tree of n_nodes 8-byte nodes
  * (scoot_node) in shared memory, as a forest walk does (1 <= n_nodes <=
  * 12288): 256 * blocks * steps node visits.  sink: device float [blocks]
- * (receives nothing in practice; it keeps the work live).  Asynchronous. */
+ * (receives nothing in practice; it keeps the work live).
+ * scoot_probe_math: y[i] of x[i] (n values, device) by one of the functions
+ * that the kernels use in place of exact ones: which = 0 the square root of a
+ * float (from 0 on), 1 exp(-x) of a float x >= 0, 2 the reciprocal of a double
+ * (2^-1000 to 2^1000), 3 the reciprocal square root of a double > 0.
+ * Asynchronous. */
 scoot_status scoot_probe_fma(scoot_ctx* ctx, int32_t packed, int32_t blocks, int32_t iters, float* sink,
                              void* stream);
+scoot_status scoot_probe_math(scoot_ctx* ctx, int32_t which, const void* x, void* y, int64_t n, void* stream);
 scoot_status scoot_probe_gather(scoot_ctx* ctx, int32_t n_nodes, int32_t blocks, int32_t steps, float* sink,
                                 void* stream);
 

@@ -17,9 +17,12 @@
 
 #include <cooperative_groups.h>
 
+#include "approx.cuh"
 #include "internal.h"
 
 namespace {
+
+using namespace scoot_dev;
 
 constexpr int kFeatThreads = 128;
 constexpr int kKmatThreads = 128;
@@ -52,22 +55,6 @@ struct GpPrepArgs {
 };
 
 __device__ __forceinline__ int64_t tri_idx(int i, int k) { return (int64_t)i * (i + 1) / 2 + k; }
-
-// 1 / sqrt(v) for v > 0 by Newton-Raphson on f(y) = 1 / y^2 - v from an
-// fp32 estimate, y <- y + y (1 - v y^2) / 2: each step doubles the correct
-// bits (24 -> 48 -> beyond fp64), in fused multiply-adds only, which keeps
-// the pivot off the slow fp64 division and square root.  Outside the fp32
-// range of the estimate the library's division and square root are used.
-__device__ __forceinline__ double rsqrt_newton(double v) {
-    if (!(v > 1e-30 && v < 1e30)) return 1.0 / sqrt(v);
-    double y = (double)rsqrtf((float)v);
-    const double h = 0.5 * v;
-    for (int it = 0; it < 3; ++it) {
-        const double e = fma(-h * y, y, 0.5);  // (1 - v y^2) / 2
-        y = fma(y, e, y);
-    }
-    return y;
-}
 
 __device__ __forceinline__ double matern_dev(double r, int kernel) {
     if (kernel == SCOOT_MATERN32) {
@@ -328,22 +315,6 @@ inline int64_t cluster_own(int n) {
         if (e > own) own = e;
     }
     return own;
-}
-
-// 1 / v for a normal v > 0 by Newton-Raphson from the hardware's estimate
-// (2^-20, then 2^-40, then beyond 53 bits): four dependent multiply-adds.
-__device__ __forceinline__ double rcp_newton(double v) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
-    y = fma(fma(-v, y, 1.0), y, y);
-    return fma(fma(-v, y, 1.0), y, y);
-}
-
-// Whether v lies in [2^-1000, 2^1000), on the integer pipes: a pivot that
-// can be inverted (a covariance's pivots lie far inside).
-__device__ __forceinline__ bool good_pivot(double v) {
-    const int hi = __double2hiint(v);
-    return hi >= ((1023 - 1000) << 20) && hi < ((1023 + 1000) << 20);
 }
 
 // What the eliminations of a block's pivots need of the pivot rows.

@@ -6,8 +6,10 @@
 //  - probe_gather: dependent walks through an array of 8-byte nodes in
 //    shared memory, one walk per thread, each step one node load whose index
 //    depends on the previous node and the walker's feature vector, the
-//    access pattern of the forest kernel's tree walks: its node-visit peak.
+//    access pattern of the forest kernel's tree walks: its node-visit peak;
+//  - probe_math: the functions of approx.cuh, value by value.
 // Results land in `sink` so that no chain is dead code.
+#include "approx.cuh"
 #include "device_common.cuh"
 #include "internal.h"
 
@@ -79,9 +81,31 @@ __global__ void __launch_bounds__(256) probe_gather(int n_nodes, int steps, uint
     if (node == seed) sink[blockIdx.x] = (float)visits;
 }
 
+__global__ void __launch_bounds__(256) probe_math(int which, const void* x, void* y, int64_t n) {
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+        if (which < 2) {
+            const float v = static_cast<const float*>(x)[i];
+            static_cast<float*>(y)[i] = which == 0 ? scoot_dev::sqrt_acc(v) : scoot_dev::exp_acc(v);
+        } else {
+            const double v = static_cast<const double*>(x)[i];
+            static_cast<double*>(y)[i] = which == 2 ? scoot_dev::rcp_newton(v) : scoot_dev::rsqrt_newton(v);
+        }
+    }
+}
+
 }  // namespace
 
 extern "C" {
+
+scoot_status scoot_probe_math(scoot_ctx* ctx, int32_t which, const void* x, void* y, int64_t n, void* stream) {
+    scoot_status s = scoot_enter(ctx);
+    if (s != SCOOT_OK) return s;
+    if (which < 0 || which > 3 || n < 1 || !x || !y) return scoot_fail(ctx, SCOOT_EINVAL, "bad probe arguments");
+    const int64_t blocks = (n + 255) / 256;
+    probe_math<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, static_cast<cudaStream_t>(stream)>>>(which, x, y, n);
+    SCOOT_LAUNCHED(ctx);
+    return SCOOT_OK;
+}
 
 scoot_status scoot_probe_fma(scoot_ctx* ctx, int32_t packed, int32_t blocks, int32_t iters, float* sink,
                              void* stream) {

@@ -94,6 +94,7 @@ _PROTOS = {
     "scoot_ctx_set_timing": [_vp, _i32],
     "scoot_ctx_set_tensor_cores": [_vp, _i32],
     "scoot_probe_fma": [_vp, _i32, _i32, _i32, _vp, _vp],
+    "scoot_probe_math": [_vp, _i32, _vp, _vp, _i64, _vp],
     "scoot_probe_gather": [_vp, _i32, _i32, _i32, _vp, _vp],
     "scoot_ctx_phase_times": [_vp, _i32, _vp, _vp, C.POINTER(_i32)],
     "scoot_prune": [_vp, _vp, _i32, _vp, _i32, _vp, _i64, _i64, _vp, _vp, _vp],
@@ -265,6 +266,13 @@ def scoot_probe_fma(ctx, packed: bool, blocks: int, iters: int, sink, stream=Non
     import torch
     _check(lib().scoot_probe_fma(_h(ctx), int(bool(packed)), int(blocks), int(iters),
                                  _dev(sink, torch.float32, "sink"), _stream(stream)), "scoot_probe_fma", _h(ctx))
+
+
+def scoot_probe_math(ctx, which: int, x, y, stream=None) -> None:
+    import torch
+    dtype = torch.float32 if which < 2 else torch.float64
+    _check(lib().scoot_probe_math(_h(ctx), int(which), _dev(x, dtype, "x"), _dev(y, dtype, "y"), int(x.numel()),
+                                  _stream(stream)), "scoot_probe_math", _h(ctx))
 
 
 def scoot_probe_gather(ctx, n_nodes: int, blocks: int, steps: int, sink, stream=None) -> None:
