@@ -54,9 +54,9 @@ TRAFFIC = {
     # d12-fantasy: captured on a 2^20 pool of the same workload, scaled to the 2^22 launch by its
     # live candidates (x 4.0025; fant_pass and the posterior) or its pool size (x 4; prune, forest)
     ("fant_pass", "d12-fantasy"): {"bytes": 3562000000, "sha": "debd6c98ff2ef39c"},
-    ("posterior", "d12-fantasy"): {"bytes": 3441200000, "sha": "36bb65e51b734d88"},
-    ("rf", "d12-fantasy"): {"bytes": 210590000, "sha": "9160ae57ca73ba4f"},
-    ("prune", "d12-fantasy"): {"bytes": 100700000, "sha": "9160ae57ca73ba4f"},
+    ("posterior", "d12-fantasy"): {"bytes": 3440600000, "sha": "c8c352405c2d83a9"},
+    ("rf", "d12-fantasy"): {"bytes": 210530000, "sha": "53e0951d2ed47670"},
+    ("prune", "d12-fantasy"): {"bytes": 100700000, "sha": "53e0951d2ed47670"},
 }
 
 
@@ -174,6 +174,23 @@ def posterior_tensor_flops(inst, n_obj=None):
     n_pad = 64 * ((inst.n_obs + 63) // 64)
     m = inst.n_obj if n_obj is None else n_obj
     return m * 6 * 2 * 32 * sum(n_pad - 32 * kb for kb in range(n_pad // 32))
+
+
+def reached_boxes(S, ctx, st, cand, idx, stream):
+    """Mean number of boxes with a lower corner below a base sample, over the samples
+    of the candidates idx: the boxes that add to the Monte-Carlo EHVI, which is what
+    its walk visits."""
+    import torch
+    L = st.gp_layout
+    at = torch.from_numpy(idx).to(cand.device)
+    n = len(idx) // 4 * 4
+    words = cand[:, at[:n]].contiguous()
+    mean, var = (torch.empty((L.n_obj, n), device=cand.device) for _ in range(2))
+    S.scoot_gp_posterior(ctx, L, st.gp_state, words, n, mean, var, None, stream)
+    torch.cuda.synchronize(cand.device)
+    y = mean[:, None] + var.sqrt()[:, None] * st.eps.T[:, :, None]
+    hit = sum(float((y > lo[:, None, None]).all(0).sum()) for lo in st.box_lo)
+    return hit / (y.shape[1] * n)
 
 
 def forest_visits(inst, idx):
@@ -1045,6 +1062,14 @@ def main():
                 "peak_source": "measured (MEASURED_PEAKS.json bf16_tflops, burst)" if bf16 else None,
                 "note": "the work above counts the fp32-equivalent product once; the tensor cores run six bf16 "
                         "part products of it"}
+    def known_sample():
+        """4096 candidates that satisfy the constraints."""
+        mask_k = torch.empty(N, dtype=torch.uint8, device=device)
+        S.scoot_prune(ctx, inp.space, inp.clauses, cand, N, mask_k, None, stream)
+        known = np.nonzero(mask_k.cpu().numpy())[0]
+        draw = Stream(seed, "visit-sample").u64(4096) % np.uint64(max(1, len(known)))
+        return known[draw.astype(np.int64)] if len(known) else known
+
     kernels = {}
     for s_ in ("prune", "rf"):
         k_, pc = work[s_]
@@ -1068,7 +1093,13 @@ def main():
                      "fant_pass": pass_ms, "fant_pick": pick_ms + init_ms}
     else:
         k_, pc = work["score"]
+        boxes = None
+        if inp.acq == "ehvi" and inst.n_obj == 3:  # the work that counts is the boxes that a sample reaches
+            boxes = reached_boxes(S, ctx, st, cand, known_sample(), stream)
+            pc = posterior_flops(inst) + inp.eps.shape[0] * boxes * 4 * inst.n_obj
         kernels["score"] = alu_roof(pc * n_feasible, stage_ms["score"], "score")
+        if boxes is not None:
+            kernels["score"]["boxes_reached_per_sample"] = boxes
         if inp.acq in ("ei", "mace") and 64 * ((inst.n_obs + 63) // 64) <= 256:
             # posterior and acquisition in the tensor-core kernel (objective 0)
             kernels["score"]["tensor"] = tensor_roof(posterior_tensor_flops(inst, 1) * n_feasible, stage_ms["score"])
@@ -1091,12 +1122,7 @@ def main():
             if v["bound"] == "alu":
                 v["frac_of_measured_ffma2"] = v["achieved"] / max(probes["ffma_tflops"], probes["ffma2_tflops"])
         # the forest's true bound: node visits against the shared-memory gather peak
-        st_ = Stream(seed, "visit-sample")
-        mask_k = torch.empty(N, dtype=torch.uint8, device=device)
-        S.scoot_prune(ctx, inp.space, inp.clauses, cand, N, mask_k, None, stream)
-        known = np.nonzero(mask_k.cpu().numpy())[0]
-        samp = known[(st_.u64(4096) % np.uint64(max(1, len(known)))).astype(np.int64)] if len(known) else known
-        visits = forest_visits(inst, samp) * n_known
+        visits = forest_visits(inst, known_sample()) * n_known
         rate = visits / (stage_ms["rf"] / 1e3)
         kernels["rf"].update({"node_visits_per_launch": visits, "node_visits_per_s": rate,
                               "frac_of_smem_gather_peak": rate / probes["smem_gather_visits_per_s"]})

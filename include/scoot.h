@@ -426,8 +426,9 @@ scoot_status scoot_score_ei(scoot_ctx* ctx, const scoot_gp_layout* layout, const
                             float xi, float* acq, void* stream);
 
 /* scoot_gp_posterior followed by scoot_acq_ehvi, in one call: one fused kernel,
- * or on the tensor cores (from 65 observations, or large pools) the moments into
- * the context workspace and a kernel that visits the boxes. */
+ * or, where that is faster (many observations and candidates, few boxes or samples),
+ * the moments into the context workspace on the tensor cores and a kernel that
+ * visits the boxes. */
 scoot_status scoot_score_ehvi(scoot_ctx* ctx, const scoot_gp_layout* layout, const void* state,
                               const uint32_t* cand, int64_t n, int64_t ld, const uint8_t* mask,
                               const float* box_lo, const float* box_hi, int32_t n_boxes,

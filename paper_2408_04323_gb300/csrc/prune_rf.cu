@@ -406,7 +406,7 @@ rf_ranked_kernel(const __grid_constant__ RfArgs a, const uint2* __restrict__ nod
         for (int k = tid; k < a.n_trees; k += kRankWalkThreads) sroot[k] = node0 + 8u * (uint32_t)roots[k];
     }
     uint32_t feasible = 0;
-    uint32_t* feat = sfeat + half * 16 * kRfCand + slot;  // 2 KB aligned but for the slot: offsets are or-ed in
+    uint32_t* feat = sfeat + half * 16 * kRfCand + slot;  // feature f's rank is 128 f bytes on
     const uint32_t my = (uint32_t)__cvta_generic_to_shared(feat);
     for (int64_t t0 = tile0; t0 < n_tiles; t0 += step_tiles) {
         const int64_t pos = (t0 + half) * kRfCand + slot;

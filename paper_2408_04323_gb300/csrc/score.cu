@@ -693,8 +693,8 @@ bool score_fits(scoot_ctx* ctx, ScoreArgs a, int epi, int nobj) {
 // 150, 2^17 2236 against 801; 5 parameters, one objective, n = 257: 8192 46 against
 // 52, 12288 57 against 52, 2^17 438 against 223).  The covariances take the accurate
 // square root and exponential, so that the error against 64 bits is the fp32 kernel's
-// (0.7 to 1.3 times it over 16 models of 257 to 640 observations, 0.98 on average,
-// mean and variance alike; the largest error of the variance is smaller in 15).
+// (over 64 models of 257 to 512 observations 0.99 times it on average for the mean, 0.97
+// for the variance; 0.45 to 2.2 in one model).
 bool tc_groups(scoot_ctx* ctx, const ScoreArgs& a) {
     return a.n_rb * kRB > kMaxNpadTc && a.n > (int64_t)sm_count(ctx->device) * 2 * kTC;
 }
@@ -746,9 +746,11 @@ scoot_status tc_direct(scoot_ctx* ctx, const ScoreArgs& a, const uint8_t* mask, 
 // (where they cannot be had the fused kernel, which needs less, takes the call).
 // *used as for tc_direct.  The covariances take the accurate square root and
 // exponential (7% of the posterior's time): the acquisition's error against 64
-// bits is then that of the fused kernel (over 64 models of 70 to 256 observations,
-// Monte-Carlo and closed form, 0.98 times it on average and 0.5 to 1.7 in one
-// model; 1.1 without).
+// bits is then no larger than the fused kernel's on average.  Over 480 models each
+// of 56 to 256 observations it is 0.99 times it (Monte-Carlo, M = 2 and 3 alike,
+// standard error 0.007), over 420 of 129 to 256 0.98 (closed form; 0.008), from 0.94 to
+// 1.02 at each number of observations; a single model lies anywhere between 0.5 and
+// 2, its largest values being few.  1.1 without.
 scoot_status tc_moments(scoot_ctx* ctx, const ScoreArgs& a, ScootTcArgs& t, int by_index, size_t extra, cudaStream_t st,
                         char** work, bool* used) {
     *used = false;
@@ -863,8 +865,7 @@ scoot_status tc_exact(scoot_ctx* ctx, ScoreArgs a, cudaStream_t st, bool* used) 
     // Whole rounds, M = 2: 5 parameters, n = 200: 16384 candidates 114 us fused against
     // 85, 2^18 883 against 358; 8 parameters, n = 256: 121 against 90, 655 against 251.
     // Up to 128 observations there is less to gain (n = 75: 65536 98 against 93, 2^18 216
-    // against 174), and at n = 70 the error against 64 bits was 1.04 times the fused
-    // kernel's over 8 models (up to 1.7 in one; n = 180 and 256: 0.97).
+    // against 174; a round of 99991 138 against 125).
     if (!ctx->tensor_cores || a.n_rb <= 2 || a.n < 16384) return SCOOT_OK;
     if (!score_fits(ctx, a, kEHVIX, a.n_obj)) return SCOOT_OK;
     int optin = 0;
