@@ -4,8 +4,8 @@ elimination of the identity), through the C ABI.
 Parity: the posterior computed from the device-built state meets the same
 bars against the oracle as the host-built state (variance 1e-6 + 1e-4 |o|;
 mean plus 2^-22 sum_j |k_j alpha_j|), on every workload, both kernels, with
-and without input warping, on both sides of the shared-memory limit of the
-factorisation (n = 160 / 161) and at n = 1 and the maximum, n = 640.  Consistency: the
+and without input warping, on both sides of the observations from which the
+scratch holds a second triangle (n = 160 / 161) and at n = 1 and the maximum, n = 640.  Consistency: the
 tables that involve no factorisation (feature map, scaled features, inverse
 lengthscales, scalars, warping, categorical table) equal the host's to one
 fp32 rounding of an fp64 value; alpha and L^{-1} agree with the host's to
@@ -132,9 +132,9 @@ def test_device_state_matches(S, ctx, name, kernel, warped):
 
 @pytest.mark.parametrize("n_obs", [1, 2, 7, 63, 64, 65, 160, 161, 384, 385, 640])
 def test_device_state_sizes(S, ctx, n_obs):
-    """Observation counts across tile edges, the shared-memory limit of the
-    factorisation (160 / 161), the cluster path's limit (384 / 385) and the maximum; the d8
-    space, two objectives."""
+    """Observation counts across tile edges, the size of the scratch (160 / 161), 384 / 385
+    and the maximum, which is beyond the cluster kernel's shared memory (its limit, 549 / 550, is
+    tests/test_gpu_gp_blocks.py's); the d8 space, two objectives."""
     base = make_instance("d8-ehvi2", seeds("d8-ehvi2")[0], n_cand=4096)
     from workloads.generate import draw_configs
     w = base.workload

@@ -67,8 +67,9 @@ def run(S, ctx, space, x, y, theta0, lo, hi, free, steps, lr, kernel=0):
                                            ("d10-ehvi3", 0, None), ("d12-fantasy", 0, 129), ("tiny", 0, None)])
 def test_lml_and_gradient_match_oracle(S, ctx, name, kernel, n):
     """Starts around the workload's hyperparameters, both sides of the
-    shared-memory limit (n = 128 / 129) and the global-memory path (n =
-    200); every objective."""
+    observations from which the call needs scratch (n = 128 / 129) and n = 200;
+    every objective.  (All by clusters; the other kernel and the changes in the use of
+    shared memory are tests/test_gpu_mle_cluster.py's.)"""
     inst = make_instance(name, seeds(name)[0], n_cand=16)
     n = inst.n_obs if n is None else n
     y = np.ascontiguousarray(inst.y_obs[:, :n])
